@@ -549,7 +549,8 @@ size_t workspace_layout(int dim, int n_leaves, size_t n, char* base, Workspace* 
     // control words, 256 bytes each, cleared together: the query's, then the chunk's
     w.acc = (unsigned long long*)carve(kCounterCount * sizeof(unsigned long long));
     w.gcount = (int*)carve(8 * sizeof(int));
-    w.counters = (int*)carve(kCounterCount * sizeof(int));
+    w.counters = (int*)carve(kCounterCount * sizeof(int) + sizeof(unsigned long long));
+    w.found = (unsigned long long*)(w.counters + kCounterCount);  // cleared with the counters
     w.bbox = (unsigned*)carve(8 * sizeof(unsigned));
     w.pair_cap = cap;
     w.slow_cap = slow;
@@ -620,6 +621,21 @@ static int bin_bits3(size_t n, int ppc) {
     const double cells = std::max(1.0, (double)n / std::max(1, ppc));
     const int b = (int)std::lround(std::log2(cells) / 3.0);
     return std::min(6, std::max(3, b));
+}
+
+// The exact pairs of a chunk's first walk above which its leaves take the nodes' far factor
+// beta instead of beta_leaf and the chunk is walked again.  Points in a crowd of small leaves
+// have several times the pairs of other points, and there the leaves' far terms are most
+// of the error.  Until the pair list grew, such a chunk did not fit it (96 entries a
+// point and 65536, in up to three tries of what was left), and its points were evaluated in
+// place with the leaves at beta; the line lies where that began, which the points in
+// flight (150,000) make a matter of the chunk's size too: at 1.4 lists up to 150,000
+// points, at 1.6 for 200,000, 1.9 for 300,000, 2.9 for 600,000, 3.3 for 2^20.  Measured, 14,000
+// points next to a 560-patch model, beta 6, beta_leaf 3.25 (158 pairs a point, 1.57 lists):
+// error 1.4e-5 at beta_leaf, 2.2e-6 at beta.
+static unsigned long long dense_limit(const Workspace& ws, size_t n) {
+    const double lists = std::min(3.3, std::max(1.4, 1.4 + ((double)n - 150000.0) / 300000.0));
+    return (unsigned long long)(lists * (96.0 * (double)ws.rcap + 65536.0));
 }
 
 // the kernels' parameters of one query
@@ -829,32 +845,46 @@ static gwn_status enqueue_chunk(gwn_model_s* m, const void* pts, int dtype, size
             if (prof)
                 for (int k : {1, 2, 4, 3}) GWN_CUDA_TRY(cudaEventRecord(ev[k], st));
         } else {
-            auto wide_pass = [&](bool list, unsigned blocks, const int* idx, const int* n_dev) {
+            const unsigned long long limit = dense_limit(ws, n);
+            const bool may_dense = m->tree.leaf_far && p.beta2_leaf < p.beta2 &&
+                                   (unsigned long long)n * (unsigned long long)m->host.n_leaves > limit;
+            const Dense none{nullptr, 0}, dense{may_dense ? ws.found : nullptr, limit};
+            auto wide_pass = [&](bool list, unsigned blocks, const int* idx, const int* n_dev, Dense d, bool again) {
                 auto k = p.work ? (list ? (o3 ? k_wide3<true, true, true> : k_wide3<false, true, true>)
                                         : (o3 ? k_wide3<true, true, false> : k_wide3<false, true, false>))
                                 : (list ? (o3 ? k_wide3<true, false, true> : k_wide3<false, false, true>)
                                         : (o3 ? k_wide3<true, false, false> : k_wide3<false, false, false>));
                 k<<<blocks, B, 0, st>>>(m->tree, ws.spos, ni, idx, n_dev, p.beta2, p.beta2_leaf, ws, ws.pairs2,
-                                        ws.slow_cap, list ? ws.olist : ws.olist2, p.work);
+                                        ws.slow_cap, list ? ws.olist : ws.olist2, p.work, d, again);
+            };
+            auto packet_pass = [&](Dense d, bool again) {
+                auto trav = p.work ? (o3 ? k_trav3<true, true> : k_trav3<false, true>)
+                                   : (o3 ? k_trav3<true, false> : k_trav3<false, false>);
+                trav<<<dim3(packets, (unsigned)m->cut_size[level]), 32, trav3_smem(m->stack_depth), st>>>(
+                    m->tree, ws.spos, ni, p.beta2, again ? p.beta2 : p.beta2_leaf, m->stack_depth, m->cuts[level], ws,
+                    p.work, ws.olist, d, again);
             };
             auto eval_pass = [&]() {
                 k_pair_eval<float><<<(unsigned)(sms * kEvalBlocks), B, 0, st>>>(m->tree, ws.spos, ws.slow_cap, ws.counters + 8,
                                                                ws.counters, ws.pairs2, ws.wacc, ws.st, ws.pairs64, ni,
                                                                p.work);
             };
+            const unsigned wide_blocks =
+                (unsigned)std::min(std::max((n + 3) / 4, std::min(n, (size_t)sms)), (size_t)sms * 16);
             if (wide) {
-                wide_pass(true, (unsigned)std::min(std::max((n + 3) / 4, std::min(n, (size_t)sms)), (size_t)sms * 16), nullptr,
-                          nullptr);
+                wide_pass(true, wide_blocks, nullptr, nullptr, none, false);
             } else if (local) {
                 auto trav = m->stack_depth <= 64 ? k_trav3_local<64>
                                                  : m->stack_depth <= 96 ? k_trav3_local<96> : k_trav3_local<128>;
                 trav<<<nb, B, 0, st>>>(m->tree, ws.spos, ni, nullptr, p.beta2, p.beta2_leaf, ws, p.work, nullptr,
                                        ws.olist, p.kappa2);
             } else {
-                auto trav = p.work ? (o3 ? k_trav3<true, true> : k_trav3<false, true>)
-                                   : (o3 ? k_trav3<true, false> : k_trav3<false, false>);
-                trav<<<dim3(packets, (unsigned)m->cut_size[level]), 32, trav3_smem(m->stack_depth), st>>>(
-                    m->tree, ws.spos, ni, p.beta2, p.beta2_leaf, m->stack_depth, m->cuts[level], ws, p.work, ws.olist);
+                packet_pass(none, false);
+            }
+            if (may_dense) {
+                k_dense_reset<<<std::min(nb, (unsigned)sms * 4), B, 0, st>>>(ws, ni, dense);
+                if (wide) wide_pass(true, wide_blocks, nullptr, nullptr, dense, true);
+                else packet_pass(dense, true);
             }
             if (prof)
                 for (int k : {1, 2}) GWN_CUDA_TRY(cudaEventRecord(ev[k], st));
@@ -875,7 +905,7 @@ static gwn_status enqueue_chunk(gwn_model_s* m, const void* pts, int dtype, size
             if (may_overflow) {
                 // the points whose pairs did not fit the list, one warp each, without a list
                 k_next_round<<<1, 32, 0, st>>>(ws);
-                wide_pass(false, (unsigned)(sms * 8), ws.olist, ws.counters + 5);
+                wide_pass(false, (unsigned)(sms * 8), ws.olist, ws.counters + 5, dense, false);
                 eval_pass();
             }
             GWN_CUDA_TRY(cudaGetLastError());
@@ -1518,7 +1548,8 @@ gwn_status noalloc_3d(gwn_model_s* m, const QueryParams& p, const void* points, 
                                               nullptr);
         (o3 ? k_wide3<true, false, false> : k_wide3<false, false, false>)
             <<<(unsigned)std::min(((size_t)c + 3) / 4, (size_t)sms * 16), B, 0, st>>>(
-                m->tree, ws.spos, c, nullptr, nullptr, p.beta2, p.beta2_leaf, ws, ws.pairs2, ws.slow_cap, ws.olist2, nullptr);
+                m->tree, ws.spos, c, nullptr, nullptr, p.beta2, p.beta2_leaf, ws, ws.pairs2, ws.slow_cap, ws.olist2, nullptr,
+                Dense{nullptr, 0}, false);
         k_pair_eval<float><<<(unsigned)(sms * kEvalBlocks), B, 0, st>>>(m->tree, ws.spos, ws.slow_cap, ws.counters + 8, ws.counters,
                                                               ws.pairs2, ws.wacc, ws.st, ws.pairs64, c, nullptr);
         k_pair_eval64_warp<float><<<(unsigned)(sms * 2), B, 0, st>>>(m->tree, ws.spos, c, ws.counters, ws.pairs64, ws.wacc,

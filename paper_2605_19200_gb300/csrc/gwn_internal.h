@@ -214,6 +214,13 @@ constexpr size_t kParts2 = (size_t)1 << 21;      // subtrees x points of a 2D ch
 constexpr uint32_t kPairOverflow = 0x100u;       // internal status bit: the point's pairs did not fit a list
 constexpr int kCounterCount = 16;                // device counters of one chunk
 
+// Whether a chunk's points have so many exact pairs that its leaves take the nodes' far
+// factor (dense_limit in gwn_api.cu); found == nullptr: never.
+struct Dense {
+    const unsigned long long* found;  // pairs of the chunk's first walk
+    unsigned long long limit;
+};
+
 // The points of one FP64 repair pass and its scratch.  The list holds point
 // indices into the arrays the repair kernels are given; count may exceed cap
 // (entries past cap were not stored and are not repaired by this pass).
@@ -260,6 +267,7 @@ struct Workspace {
                       // [7] pairs of the first pass, [8] pairs left to the full evaluator in this pass,
                       // [9] the same in the first pass, [10] repair pairs the FP64 tables left,
                       // [11] padding entries of the pair list
+    unsigned long long* found;  // (point, leaf) pairs that the chunk's first walk needs exactly, listed or not
     int* olist;       // n: points whose pairs did not fit in the first pass
     int* olist2;      // n: in the second
     unsigned long long* work;  // kWorkCount counters

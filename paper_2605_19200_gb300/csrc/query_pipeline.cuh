@@ -269,6 +269,18 @@ __device__ __forceinline__ void flush_packet_pairs(const int2* buf, const unsign
     }
 }
 
+__device__ __forceinline__ bool is_dense(Dense d) { return d.found && *d.found > d.limit; }
+
+// before a dense chunk's second walk: what the first one left
+__global__ void k_dense_reset(Workspace ws, int n, Dense d) {
+    if (!is_dense(d)) return;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        ws.wacc[i] = 0.f;
+        ws.st[i] = 0u;
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) ws.counters[0] = ws.counters[3] = ws.counters[11] = 0;
+}
+
 // bytes of dynamic shared memory of k_trav3 (one warp) with a stack of `depth` entries
 inline size_t trav3_smem(int depth) { return (size_t)depth * 12 + kPairBuf * (sizeof(int2) + 1); }
 
@@ -304,12 +316,14 @@ inline size_t trav3_smem(int depth) { return (size_t)depth * 12 + kPairBuf * (si
 // their sums.
 // depth: entries of the warp stack (pending near siblings along the packet's
 // path), chosen per model from its tree depth.  O3: the model evaluates the
-// order-3 terms; COUNT: work counters (instances of their own, for the registers)
+// order-3 terms; COUNT: work counters (instances of their own, for the registers).
+// again: the second walk of a dense chunk (d), nothing where the chunk is not dense
 template <bool O3, bool COUNT>
 __global__ void __launch_bounds__(32, 28) k_trav3(DevTree t, const float4* spos, int n, float beta2, float beta2l,
                                                   int depth, TreeCut cut, Workspace ws, unsigned long long* work,
-                                                  int* olist_out) {
+                                                  int* olist_out, Dense d, bool again) {
     extern __shared__ int2 sdyn[];
+    if (again && !is_dense(d)) return;
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x;
     const unsigned lbit = 1u << lane;
@@ -331,6 +345,7 @@ __global__ void __launch_bounds__(32, 28) k_trav3(DevTree t, const float4* spos,
     float w0 = 0.f, w1 = 0.f;
     uint32_t st0 = 0, st1 = 0;
     int bcnt = 0, npad = 0;            // warp-uniform: entries in buf, padding entries so far
+    unsigned nfound = 0;               // warp-uniform: exact pairs
     unsigned ovf0 = 0, ovf1 = 0;       // queries with pairs that did not fit the list
     int sp = 0;                        // warp-uniform
     const float b2l = t.leaf_far ? beta2l : INFINITY;
@@ -383,6 +398,7 @@ __global__ void __launch_bounds__(32, 28) k_trav3(DevTree t, const float4* spos,
                     own[bcnt + nn] = 64;
                 }
                 npad += even - nn;
+                nfound += nn;
                 bcnt += even;
             }
             m0 = m1 = 0u;
@@ -438,6 +454,7 @@ __global__ void __launch_bounds__(32, 28) k_trav3(DevTree t, const float4* spos,
     __syncwarp();
     flush_packet_pairs(buf, own, bcnt, ws, ovf0, ovf1);
     if (lane == 0 && npad) atomicAdd(&ws.counters[11], npad);
+    if (lane == 0 && nfound && !again) atomicAdd(ws.found, (unsigned long long)nfound);
     if (ovf0 & lbit) st0 |= kPairOverflow;
     if (ovf1 & lbit) st1 |= kPairOverflow;
     auto put = [&](int q, float w, uint32_t st) {
@@ -495,6 +512,7 @@ __global__ void __launch_bounds__(128) k_trav3_local(DevTree t, const float4* sp
     float w = 0.f;
     uint32_t st = 0;
     int bcnt = 0;                      // warp-uniform: entries in buf
+    unsigned nfound = 0;               // warp-uniform: exact pairs
     unsigned ovf = 0;                  // lanes with pairs that did not fit the list
     int sp = 0;                        // warp-uniform
     const unsigned amask = __ballot_sync(full, active);
@@ -584,6 +602,7 @@ __global__ void __launch_bounds__(128) k_trav3_local(DevTree t, const float4* sp
                     buf[pos] = make_int2(qi, li);
                     own[pos] = (unsigned char)lane;
                 }
+                nfound += nn;
                 bcnt += nn;
             }
             return 0u;
@@ -647,6 +666,7 @@ __global__ void __launch_bounds__(128) k_trav3_local(DevTree t, const float4* sp
         ws.st[qi] = st;
         if (st & kPairOverflow) olist_out[atomicAdd(&ws.counters[3], 1)] = qi;
     }
+    if (lane == 0 && nfound) atomicAdd(ws.found, (unsigned long long)nfound);
     if (work) flush_work(wl, work);
 }
 
@@ -664,12 +684,15 @@ __global__ void __launch_bounds__(128) k_trav3_local(DevTree t, const float4* sp
 // query one after the other are the longest chain.
 // A query costs about twice the instructions of its share of a packet, with 64
 // times the warps.
-// list, n_dev: as in k_trav3 (n_dev: the list's length on the device)
+// list, n_dev: as in k_trav3 (n_dev: the list's length on the device); again: as in
+// k_trav3, without it a dense chunk's leaves take beta2
 constexpr int kWideStack = 768;
 template <bool O3, bool COUNT, bool LIST>
 __global__ void __launch_bounds__(128) k_wide3(DevTree t, const float4* spos, int n, const int* list, const int* n_dev,
                                                float beta2, float beta2l, Workspace ws, int2* slow, long long slow_cap,
-                                               int* olist_out, unsigned long long* work) {
+                                               int* olist_out, unsigned long long* work, Dense d,
+                                               bool again) {
+    if (again && !is_dense(d)) return;
     __shared__ int sstk[4][kWideStack];
     __shared__ int sfar[4][96], sleaf[4][128];
     __shared__ float4 slfar[LIST ? 1 : 4][LIST ? 1 : 128];
@@ -680,7 +703,7 @@ __global__ void __launch_bounds__(128) k_wide3(DevTree t, const float4* spos, in
     int *stk = sstk[wid], *fq = sfar[wid], *lq = sleaf[wid];
     WorkLocal wl = {};
     if (n_dev) n = *n_dev;
-    const float b2l = t.leaf_far ? beta2l : INFINITY;
+    const float b2l = t.leaf_far ? (is_dense(d) ? beta2 : beta2l) : INFINITY;
     const float ratio2 = kRatio32 * kRatio32, inv4pi = 0.07957747154594767f;
     int npair = 0;
     // few points: a block (an SM) each first
@@ -711,6 +734,7 @@ __global__ void __launch_bounds__(128) k_wide3(DevTree t, const float4* spos, in
         };
         auto exact_leaves = [&]() {
             if (LIST) {
+                npair += nl;
                 long long base = 0;
                 if (lane == 0 && nl) base = list_slots(&ws.counters[0], nl, ws.pair_cap);
                 base = __shfl_sync(full, base, 0);
@@ -826,6 +850,7 @@ __global__ void __launch_bounds__(128) k_wide3(DevTree t, const float4* spos, in
         __syncwarp();
     }
     if (!LIST && lane == 0 && npair) atomicAdd(&ws.counters[0], npair);
+    if (LIST && !again && lane == 0 && npair) atomicAdd(ws.found, (unsigned long long)npair);
     if (COUNT) flush_work(wl, work);
 }
 
