@@ -513,7 +513,8 @@ size_t workspace_layout(int dim, int n_leaves, size_t n, char* base, Workspace* 
                                    : std::max((long long)n * 128 + 65536,
                                               dim == 3 ? std::min((long long)n * n_leaves, 1ll << 26) & ~1ll : 0ll);
     const size_t cells = kMaxBinCells;  // the finest binning of either dimension
-    const size_t hist = cells + kMaxBinCells / kScanTile;  // and the scan's tile sums
+    const size_t hist = std::max(cells + kMaxBinCells / kScanTile,  // and the scan's tile sums
+                                 (size_t)n_leaves);                // k_few_sort: an entry per leaf
     const size_t keyn = n;
     size_t off = 0;
     auto carve = [&](size_t bytes) {
@@ -718,7 +719,7 @@ static gwn_status enqueue_repair(gwn_model_s* m, const QueryParams& p, const voi
 static gwn_status enqueue_chunk(gwn_model_s* m, const void* pts, int dtype, size_t n, size_t off, double* out_w,
                                 int* out_label, uint32_t* out_status, const gwn_query_opts& qo, cudaStream_t st,
                                 const Workspace& ws,
-                                bool local_list, bool accum) {
+                                bool local_list, bool accum, bool whole) {
     const QueryParams p = query_params(m, qo, ws);
     const int pc = m->prof_chunks;
     const bool prof = qo.profile != 0 && pc < gwn_model_s::kMaxProfChunks;
@@ -784,6 +785,7 @@ static gwn_status enqueue_chunk(gwn_model_s* m, const void* pts, int dtype, size
         // 1. spatial binning of the points (counting sort by Morton cell)
         const bool o3 = m->tree.order3 != 0;
         const bool local = !o3 && p.kappa2 > 0.f;  // packets take far nodes by local expansion
+        const bool few = whole && m->dim == 3 && n <= (size_t)kFewPoints;  // few3d.cuh
         const bool wide = m->dim == 3 && !direct3 && !local && n <= kWideMaxPoints;  // one warp per point: their order does not matter
         const int* key = nullptr;
         if (n >= 2048 && !wide) {
@@ -811,19 +813,56 @@ static gwn_status enqueue_chunk(gwn_model_s* m, const void* pts, int dtype, size
             // every leaf for every point, the leaves in slices until the blocks fill the GPU
             const unsigned slices = (unsigned)std::max<long long>(
                 1, std::min<long long>(std::min<long long>(m->host.n_leaves, 65535), ((long long)sms * 16 + nb - 1) / nb));
-            GWN_CUDA_TRY(cudaMemsetAsync(ws.rw, 0, n * sizeof(double), st));
-            k_direct3<<<dim3(nb, slices), B, 0, st>>>(m->tree, ws.spos, ni, ws.rw, ws.st, ws.counters, ws.pairs2,
-                                                      ws.slow_cap, ws.olist);
-            k_pair_eval<double><<<(unsigned)(sms * kEvalBlocks), B, 0, st>>>(m->tree, ws.spos, ws.slow_cap, ws.counters + 8,
-                                                                   ws.counters, ws.pairs2, ws.rw, ws.st, ws.pairs64, ni,
-                                                                   nullptr);
-            k_pair_eval64_warp<double><<<(unsigned)(sms * 2), B, 0, st>>>(m->tree, ws.spos, ni, ws.counters, ws.pairs64,
-                                                                          ws.rw, ws.st);
-            if ((long long)n * m->host.n_leaves > ws.slow_cap)
-                k_direct_overflow3<<<(unsigned)(sms * 4), B, 0, st>>>(m->tree, ws.spos, ws.rw, ws.st, ws.counters, ws.olist);
+            float* few_val = reinterpret_cast<float*>(ws.rpairs);  // the repair's pairs come later
+            if (few && (long long)n * m->host.n_leaves <= 2 * kRepairPairCap) {
+                k_few_direct<<<(unsigned)(sms * 8), B, 0, st>>>(m->tree, ws.spos, ni, few_val, ws.st);
+                k_few_direct_sum<<<1, 32 * kFewPoints, 0, st>>>(ni, m->host.n_leaves, few_val, ws.rw);
+            } else {
+                GWN_CUDA_TRY(cudaMemsetAsync(ws.rw, 0, n * sizeof(double), st));
+                k_direct3<<<dim3(nb, slices), B, 0, st>>>(m->tree, ws.spos, ni, ws.rw, ws.st, ws.counters, ws.pairs2,
+                                                          ws.slow_cap, ws.olist);
+                k_pair_eval<double><<<(unsigned)(sms * kEvalBlocks), B, 0, st>>>(m->tree, ws.spos, ws.slow_cap, ws.counters + 8,
+                                                                       ws.counters, ws.pairs2, ws.rw, ws.st, ws.pairs64, ni,
+                                                                       nullptr);
+                k_pair_eval64_warp<double><<<(unsigned)(sms * 2), B, 0, st>>>(m->tree, ws.spos, ni, ws.counters, ws.pairs64,
+                                                                              ws.rw, ws.st);
+                if ((long long)n * m->host.n_leaves > ws.slow_cap)
+                    k_direct_overflow3<<<(unsigned)(sms * 4), B, 0, st>>>(m->tree, ws.spos, ws.rw, ws.st, ws.counters, ws.olist);
+            }
             // every point to repair goes to the chunk's own list (repaired by the direct sum below)
             k_finish<double><<<nb, B, 0, st>>>(ni, ws.spos, ws.rw, ws.st, p.precision, p.band, out_w, out_label, out_status,
                                                ws.rlist, rcount, (int)off, ws.rlist_g, ws.gcount, 0);
+            GWN_CUDA_TRY(cudaGetLastError());
+        } else if (few) {
+            // one packet's walk, its pairs sorted by leaf into the near pairs' place; these take the list's
+            const long long few_cap = ws.slow_cap;
+            Workspace fw = ws;
+            fw.pair_cap = few_cap;
+            if (prof) GWN_CUDA_TRY(cudaEventRecord(ev[0], st));
+            if (local) {
+                auto trav = m->stack_depth <= 64 ? k_trav3_local<64>
+                                                 : m->stack_depth <= 96 ? k_trav3_local<96> : k_trav3_local<128>;
+                trav<<<1, B, 0, st>>>(m->tree, ws.spos, ni, nullptr, p.beta2, p.beta2_leaf, fw, p.work, nullptr, ws.olist,
+                                      p.kappa2);
+            } else {
+                (o3 ? k_few_walk<true> : k_few_walk<false>)<<<1, 32, 0, st>>>(m->tree, ws.spos, ni, p.beta2, p.beta2_leaf,
+                                                                            fw, p.work, ws.olist);
+            }
+            if (prof) GWN_CUDA_TRY(cudaEventRecord(ev[1], st));
+            k_few_sort<<<1, 1024, 0, st>>>(m->host.n_leaves, few_cap, ws.counters, ws.pairs, ws.hist, ws.pairs2);
+            if (prof) GWN_CUDA_TRY(cudaEventRecord(ev[2], st));
+            k_few_fast<<<(unsigned)(sms * 16), B, 0, st>>>(m->tree, ws.spos, few_cap, ws.counters, ws.pairs2, ws.wacc,
+                                                           ws.st, ws.pairs, p.work);
+            if (prof) GWN_CUDA_TRY(cudaEventRecord(ev[4], st));
+            k_few_eval<<<(unsigned)(sms * 8), B, 0, st>>>(m->tree, ws.spos, ws.counters, ws.pairs, ws.wacc, ws.st,
+                                                          ws.pairs64, ni, p.work);
+            if (prof) GWN_CUDA_TRY(cudaEventRecord(ev[3], st));
+            k_pair_eval64_warp<float><<<(unsigned)(sms * 2), B, 0, st>>>(m->tree, ws.spos, ni, ws.counters, ws.pairs64,
+                                                                         ws.wacc, ws.st);
+            if ((long long)n * m->host.n_leaves > few_cap)
+                k_overflow3<<<1, B, 0, st>>>(m->tree, ws.spos, p.beta2, ws, ws.olist);
+            k_finish<float><<<nb, B, 0, st>>>(ni, ws.spos, ws.wacc, ws.st, p.precision, p.band, out_w, out_label, out_status,
+                                              ws.rlist, rcount, (int)off, ws.rlist_g, ws.gcount, ws.rcap);
             GWN_CUDA_TRY(cudaGetLastError());
         } else {
         // 2. traversal
@@ -963,7 +1002,7 @@ gwn_status gwn_enqueue_device(gwn_model_s* m, const void* pts, int dtype, size_t
         else GWN_CUDA_TRY(cudaMemsetAsync(ws.counters, 0, 2 * kControlBytes, st));
         gwn_status s = enqueue_chunk(m, reinterpret_cast<const char*>(pts) + off * esz, dtype, c, off, out_w + off,
                                      out_label ? out_label + off : nullptr, out_status ? out_status + off : nullptr,
-                                     qo, st, ws, local, !(repair && off + c == n));
+                                     qo, st, ws, local, !(repair && off + c == n), c == n);
         if (s != GWN_OK) return s;
     }
     // one FP64 repair pass over the points that every chunk listed (indices into

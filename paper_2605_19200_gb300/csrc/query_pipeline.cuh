@@ -670,6 +670,10 @@ __global__ void __launch_bounds__(128) k_trav3_local(DevTree t, const float4* sp
     if (work) flush_work(wl, work);
 }
 
+}  // namespace gwn
+#include "few3d.cuh"  // the packet walk and pair kernels of a handful of points
+namespace gwn {
+
 // One warp per query: the traversal and the far exact leaves of a query spread over
 // the lanes.  Used for few points, where a packet's walk (one node at a time) and
 // the later stages are all latency, and for the points whose pairs did not fit

@@ -38,3 +38,45 @@ def test_crowded_leaves_take_the_nodes_far_factor(n):
     assert not torch.any(st & gwn.QS_STACK_OVERFLOW)
     wb, _, _ = m.query(pts, beta_leaf=9.0)
     assert float((w - wb).abs().max()) <= 5e-6
+
+
+def _cube():
+    """A closed cube: its winding number is 0 outside."""
+    from synth import geometry as G
+    out = []
+    for ax in range(3):
+        a, b = np.zeros(3), np.zeros(3)
+        a[(ax + 1) % 3] = b[(ax + 2) % 3] = 1
+        for s in (0, 1):
+            o = np.zeros(3)
+            o[ax] = s
+            out.append(G.planar_patch(o, a, b) if s else G.planar_patch(o, b, a))
+    return out
+
+
+# values outside the cube, all of them truncation and rounding, in the order of sums that queries
+# of a handful of points keep: (order, points, mode) -> values
+_OUTSIDE = {
+    (2, 7, gwn.MODE_BVH): [-2.60828383e-05, -5.96280097e-06, 1.08491986e-05, 2.28533008e-05, 6.47999987e-05,
+                           -7.4230461e-06, -1.07851747e-05],
+    (3, 1, gwn.MODE_BVH): [0.000139282085],
+    (3, 7, gwn.MODE_BVH): [1.36382878e-05, 9.608455e-06, 8.14069062e-06, 2.05226243e-05, -8.98176804e-05,
+                           -6.27432019e-06, -1.46380626e-06],
+    (2, 7, gwn.MODE_DIRECT): [2.92038749e-09, -2.00088834e-09, 2.31011654e-10, 3.81987775e-11, 3.97267286e-09,
+                              3.53975338e-09, 6.34463504e-09],
+}
+
+
+@pytest.mark.parametrize("order,n,mode", list(_OUTSIDE))
+def test_few_points_keep_their_values(order, n, mode):
+    """Values next to 0, pinned to 2e-5 of their norm (the bound an FP32 output is held to)."""
+    b, bl = {2: (6.0, 3.25), 3: (4.5, 3.0)}[order]
+    m = gwn.gwn_build_3d(_cube(), beta=b, beta_leaf=bl, order=order)
+    r = np.random.default_rng(n + order)
+    d = r.normal(size=(n, 3))
+    d /= np.max(np.abs(d), axis=1, keepdims=True)
+    q = (0.5 + d * r.uniform(0.55, 1.0, (n, 1))).astype(np.float32)
+    ref = np.array(_OUTSIDE[order, n, mode])
+    w = np.stack([m.query(torch.from_numpy(q).cuda(), mode=mode)[0].cpu().numpy() for _ in range(5)])
+    off = np.linalg.norm(w - ref, axis=1) / np.linalg.norm(ref)
+    assert np.median(off) <= 2e-5  # pairs' sums are atomic: one run's order may differ
