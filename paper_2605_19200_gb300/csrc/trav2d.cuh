@@ -41,6 +41,48 @@ GWN_HD inline T far2_harm(const T* h, T rx, T ry, T i2) {
     return x * vr - y * vi;
 }
 
+// exact FP64 value of leaf li for a q outside its box, as the complex number whose
+// argument is its angle; false inside the box
+GWN_HD inline bool leaf2_chord64(const double* L, double qx, double qy, double& dot, double& cross) {
+    if (!(L[0] > qx || L[1] < qx || L[2] > qy || L[3] < qy)) return false;
+    const double ax = L[4] - qx, ay = L[5] - qy, bx = L[6] - qx, by = L[7] - qy;
+    cross = ax * by - ay * bx;
+    dot = ax * bx + ay * by;
+    return true;
+}
+
+// The FP64 sum of leaf angles with one arc tangent for four leaves: an angle of at most
+// atan(0.9) = 41.99 degrees multiplies the running complex number (the product's argument stays
+// below 168 degrees, far from the cut at 180, where rounding would decide the sign:
+// leaves of exactly 45 degrees are what halved sides of a square show its centre), larger
+// ones take their own.  An FP64 atan2 is about a hundred instructions on a pipe that runs at
+// 1/64 of the FP32 rate, a product four.
+struct Angle64 {
+    double re = 1.0, im = 0.0, sum = 0.0;
+    double w = 0.0;  // values that are not angles
+    int n = 0;
+    GWN_HD inline void add(double dot, double cross) {
+        if (fabs(cross) <= 0.9 * dot) {
+            const double r = re * dot - im * cross;
+            im = re * cross + im * dot;
+            re = r;
+            if (++n == 4) flush();
+        } else {
+            sum += atan2(cross, dot);
+        }
+    }
+    GWN_HD inline void flush() {
+        if (n) sum += atan2(im, re);
+        re = 1.0;
+        im = 0.0;
+        n = 0;
+    }
+    GWN_HD inline double value() {  // GWN of the leaves added
+        flush();
+        return w + sum * Num<double>::inv2pi;
+    }
+};
+
 #if defined(__CUDACC__)
 __device__ __forceinline__ f32x2 dup2(float a) { return pack2(a, a); }
 
@@ -269,46 +311,6 @@ __device__ __forceinline__ float value2(const float* part, const long long* near
     const long long v = near[q];
     return v ? w + (float)((double)v * (1.0 / (double)kNearUnit)) : w;
 }
-
-// exact FP64 value of leaf li for a q outside its box, as the complex number whose
-// argument is its angle; false inside the box
-__device__ __forceinline__ bool leaf2_chord64(const double* L, double qx, double qy, double& dot, double& cross) {
-    if (!(L[0] > qx || L[1] < qx || L[2] > qy || L[3] < qy)) return false;
-    const double ax = L[4] - qx, ay = L[5] - qy, bx = L[6] - qx, by = L[7] - qy;
-    cross = ax * by - ay * bx;
-    dot = ax * bx + ay * by;
-    return true;
-}
-
-// The FP64 sum of leaf angles with one arc tangent for four leaves: an angle below 45
-// degrees multiplies the running complex number (the product's argument stays below
-// 180 degrees), larger ones take their own.  An FP64 atan2 is about a hundred
-// instructions on a pipe that runs at 1/64 of the FP32 rate, a product four.
-struct Angle64 {
-    double re = 1.0, im = 0.0, sum = 0.0;
-    double w = 0.0;  // values that are not angles
-    int n = 0;
-    __device__ __forceinline__ void add(double dot, double cross) {
-        if (fabs(cross) <= dot) {
-            const double r = re * dot - im * cross;
-            im = re * cross + im * dot;
-            re = r;
-            if (++n == 4) flush();
-        } else {
-            sum += atan2(cross, dot);
-        }
-    }
-    __device__ __forceinline__ void flush() {
-        if (n) sum += atan2(im, re);
-        re = 1.0;
-        im = 0.0;
-        n = 0;
-    }
-    __device__ __forceinline__ double value() {  // GWN of the leaves added
-        flush();
-        return w + sum * Num<double>::inv2pi;
-    }
-};
 
 // FP64 value of one leaf into the sums
 __device__ __forceinline__ void leaf2_add64(const DevTree& t, int li, double qx, double qy, Angle64& a, uint32_t& st) {

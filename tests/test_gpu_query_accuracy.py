@@ -80,3 +80,40 @@ def test_few_points_keep_their_values(order, n, mode):
     w = np.stack([m.query(torch.from_numpy(q).cuda(), mode=mode)[0].cpu().numpy() for _ in range(5)])
     off = np.linalg.norm(w - ref, axis=1) / np.linalg.norm(ref)
     assert np.median(off) <= 2e-5  # pairs' sums are atomic: one run's order may differ
+
+
+def _octants(shape, c, r, ccw, half=False):
+    """Curves that show c at 45 degrees each: a square with halved sides, a circle of eight arcs, or
+    the upper half of them."""
+    from synth import geometry as G
+    n = 4 if half else 8
+    if shape == "circle":
+        out = [G.arc(c, r, 0.25 * np.pi * k, 0.25 * np.pi * (k + 1)) for k in range(n)]
+    else:
+        v = np.array([[1, 0], [1, 1], [0, 1], [-1, 1], [-1, 0], [-1, -1], [0, -1], [1, -1], [1, 0]], dtype=float)
+        out = [G.polyline(c + r * v[k:k + 2], closed=False) for k in range(n)]
+    return out if ccw else [x.reversed() for x in out]
+
+
+@pytest.mark.parametrize("ccw", [True, False])
+@pytest.mark.parametrize("shape", ["square", "circle"])
+def test_leaves_of_45_degrees(shape, ccw):
+    """FP64 traversal, direct sum (32 copies: whole groups in each lane) and repair at the centre: whole
+    and half turns to rounding (the sums' 2^-52 per leaf, 1e-12 for 256 of them)."""
+    rng = np.random.default_rng(2)
+    sgn = 1.0 if ccw else -1.0
+    for k in range(12):
+        c = np.zeros(2) if k == 0 else rng.uniform(-1, 1, 2)
+        r = 1.0 if k == 0 else float(np.exp(rng.uniform(-1, 1)))
+        q = torch.from_numpy(c[None]).cuda()
+        for copies in (1, 32):
+            curves = [x for x in _octants(shape, c, r, ccw) for _ in range(copies)]
+            m = gwn.gwn_build_2d(curves, max_aabb_frac=0.0, beta=1e9)
+            for mode in (gwn.MODE_BVH, gwn.MODE_DIRECT):
+                w, _, _ = m.query(q, precision=gwn.PREC_FP64, mode=mode)
+                assert abs(float(w[0]) - sgn * copies) <= 1e-12 * copies
+        for kw in (dict(), dict(beta_repair=1e9)):  # a half turn goes to the repair
+            m = gwn.gwn_build_2d(_octants(shape, c, r, ccw, half=True), max_aabb_frac=0.0, beta=1e9, **kw)
+            w, _, st = m.query(q)
+            assert int(st[0]) & gwn.QS_REPAIRED
+            assert abs(float(w[0]) - 0.5 * sgn) <= 1e-12
