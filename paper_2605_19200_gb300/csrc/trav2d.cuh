@@ -11,6 +11,8 @@
 // place of atan2.
 #pragma once
 
+#include <cstring>
+
 #include "gwn_internal.h"
 #include "kernels2d.cuh"
 #include "pairs3d.cuh"
@@ -55,14 +57,18 @@ GWN_HD inline bool leaf2_chord64(const double* L, double qx, double qy, double& 
 // atan(0.9) = 41.99 degrees multiplies the running complex number (the product's argument stays
 // below 168 degrees, far from the cut at 180, where rounding would decide the sign:
 // leaves of exactly 45 degrees are what halved sides of a square show its centre), larger
-// ones take their own.  An FP64 atan2 is about a hundred instructions on a pipe that runs at
+// ones and those whose product could leave the range of a double take their own.  An FP64 atan2 is about a hundred instructions on a pipe that runs at
 // 1/64 of the FP32 rate, a product four.
 struct Angle64 {
     double re = 1.0, im = 0.0, sum = 0.0;
     double w = 0.0;  // values that are not angles
     int n = 0;
     GWN_HD inline void add(double dot, double cross) {
-        if (fabs(cross) <= 0.9 * dot) {
+        // four factors between 2^-199 and 1.35 x 2^199 stay within a double (dot's exponent: integer
+        // instructions, the FP64 pipe is the slow one)
+        unsigned long long bits;
+        memcpy(&bits, &dot, sizeof(bits));
+        if (fabs(cross) <= 0.9 * dot && (unsigned)(bits >> 52) - (1023u - 199u) < 398u) {
             const double r = re * dot - im * cross;
             im = re * cross + im * dot;
             re = r;

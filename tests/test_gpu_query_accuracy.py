@@ -117,3 +117,17 @@ def test_leaves_of_45_degrees(shape, ccw):
             w, _, st = m.query(q)
             assert int(st[0]) & gwn.QS_REPAIRED
             assert abs(float(w[0]) - 0.5 * sgn) <= 1e-12
+
+
+def test_fp64_sums_stay_finite_far_away():
+    """FP64 direct sum and traversal (every leaf exact) 1e35 to 1e70 away: outside a closed loop of 48
+    leaves.  A leaf's end points round to the same vector there, and its cross product is at most the
+    rounding of a fused one, 2^-53 of the dot product: 48 x 2^-53 / (2 pi) = 8.5e-16."""
+    from synth import geometry as G
+    curves = [G.arc((0, 0), 1.0, np.pi * k / 24, np.pi * (k + 1) / 24) for k in range(48)]
+    m = gwn.gwn_build_2d(curves, max_aabb_frac=0.0, beta=1e100)
+    d = np.array([[1.0, 0.3], [-0.4, 1.0], [-1.0, -1.0]])
+    q = np.concatenate([10.0 ** e * d for e in (35, 38, 40, 50, 70)])
+    for mode in (gwn.MODE_BVH, gwn.MODE_DIRECT):
+        w, _, _ = m.query(torch.from_numpy(q).cuda(), precision=gwn.PREC_FP64, mode=mode)
+        assert float(w.abs().max()) <= 1e-15

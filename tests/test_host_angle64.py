@@ -57,3 +57,15 @@ def test_leaves_of_45_degrees(hx, shape, ccw, copies, stride):
         if not ccw:
             p = p[::-1][:, [2, 3, 0, 1]]
         assert abs(hx(p, c, stride) - (copies if ccw else -copies)) <= 1e-13 * copies
+
+
+@pytest.mark.parametrize("e", range(-75, 80, 5))
+def test_scales(hx, e):
+    """A closed loop of 24 leaves of 15 degrees at any scale that one arc tangent per leaf holds
+    (products of coordinates above 1e-300 and below 1e300): one turn inside, none outside, to the
+    leaves' rounding (24 x 2^-52)."""
+    t = 2 * np.pi * np.arange(24) / 24
+    v = 10.0 ** e * np.stack([np.cos(t), np.sin(t)], axis=1)
+    p = np.concatenate([v, np.roll(v, -1, axis=0)], axis=1)
+    for q, w in (((0.0, 0.0), 1.0), ((0.3, -0.2), 1.0), ((3.0, 1.0), 0.0), ((1e3, 2e3), 0.0)):
+        assert abs(hx(p, 10.0 ** e * np.array(q)) - w) <= 1e-14
