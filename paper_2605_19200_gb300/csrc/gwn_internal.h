@@ -214,6 +214,18 @@ constexpr size_t kParts2 = (size_t)1 << 21;      // subtrees x points of a 2D ch
 constexpr uint32_t kPairOverflow = 0x100u;       // internal status bit: the point's pairs did not fit a list
 constexpr int kCounterCount = 16;                // device counters of one chunk
 
+// Nodes that a step takes from a stack with sp of its cap entries in use, at most width, each of
+// which may push two.  With half of the stack in use a step takes 1/32 of the free entries, at last one
+// node at a time, so that a level costs fewer and fewer entries: any tree of 100 levels fits,
+// where full steps (32 or 256 nodes a level) overflow at 24 levels of the smaller stacks.
+// 0: full.
+GWN_HD inline int stack_take(int sp, int width, int cap) {
+    const int room = cap - sp;
+    int n = 2 * room >= cap ? width : room >= 64 ? room / 32 : room > 0 ? 1 : 0;
+    if (n > width) n = width;
+    return n < sp ? n : sp;
+}
+
 // Whether a chunk's points have so many exact pairs that its leaves take the nodes' far
 // factor (dense_limit in gwn_api.cu); found == nullptr: never.
 struct Dense {

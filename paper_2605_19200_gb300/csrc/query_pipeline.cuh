@@ -690,7 +690,7 @@ namespace gwn {
 // times the warps.
 // list, n_dev: as in k_trav3 (n_dev: the list's length on the device); again: as in
 // k_trav3, without it a dense chunk's leaves take beta2
-constexpr int kWideStack = 768;
+constexpr int kWideStack = 768;  // stack_take
 template <bool O3, bool COUNT, bool LIST>
 __global__ void __launch_bounds__(128) k_wide3(DevTree t, const float4* spos, int n, const int* list, const int* n_dev,
                                                float beta2, float beta2l, Workspace ws, int2* slow, long long slow_cap,
@@ -825,8 +825,7 @@ __global__ void __launch_bounds__(128) k_wide3(DevTree t, const float4* spos, in
         test(lane == 0, t.root, t.root < 0 ? __ldg(t.lhdr + ~t.root) : __ldg(t.hdr + t.root));
         __syncwarp();
         while (sp > 0) {
-            // two children per node taken: never past the stack's end
-            const int take = min(min(sp, 32), kWideStack - sp);
+            const int take = stack_take(sp, 32, kWideStack);
             if (take <= 0) {
                 st |= GWN_QS_STACK_OVERFLOW;  // the rest is dropped, the point repaired
                 break;
@@ -1552,7 +1551,11 @@ __global__ void __launch_bounds__(32 * kRepairWarps) k_rtrav_warp(DevTree t, con
         int sp = 1;
         __syncwarp();
         while (sp > 0) {
-            const int take = min(sp, 32);
+            const int take = stack_take(sp, 32, kWarpStack);
+            if (take <= 0) {
+                st |= GWN_QS_UNRESOLVED;  // stack full: the rest is dropped (flagged)
+                break;
+            }
             const int node = lane < take ? stk[sp - 1 - lane] : 0;
             sp -= take;
             __syncwarp();
@@ -1621,13 +1624,11 @@ __global__ void __launch_bounds__(32 * kRepairWarps) k_rtrav_warp(DevTree t, con
                 if (lane >= off) incl += v;
             }
             const int total = __shfl_sync(0xffffffffu, incl, 31);
-            if (sp + total > kWarpStack) {
-                st |= GWN_QS_UNRESOLVED;  // stack full: those subtrees are dropped (flagged)
-            } else if (npush) {
+            if (npush) {
                 stk[sp + incl - 2] = c1;
                 stk[sp + incl - 1] = c0;
             }
-            if (sp + total <= kWarpStack) sp += total;
+            sp += total;
             __syncwarp();
         }
         for (int off = 16; off > 0; off >>= 1) {

@@ -394,7 +394,11 @@ __global__ void __launch_bounds__(256) k_rtrav2(DevTree t, const void* pts, int 
         int sp = 1;  // block-uniform
         __syncthreads();
         while (sp > 0) {
-            const int take = min(sp, 256);
+            const int take = stack_take(sp, 256, kBlockStack2);
+            if (take <= 0) {
+                st |= GWN_QS_UNRESOLVED;  // stack full: the rest is dropped (flagged)
+                break;
+            }
             const int node = tid < take ? stk[sp - 1 - tid] : 0;
             sp -= take;
             int2 ch = make_int2(0, 0);
@@ -421,16 +425,12 @@ __global__ void __launch_bounds__(256) k_rtrav2(DevTree t, const void* pts, int 
                 at += w < wid ? wcnt[w] : 0;
                 total += wcnt[w];
             }
-            if (sp + 2 * total > kBlockStack2) {
-                st |= GWN_QS_UNRESOLVED;  // stack full: those subtrees are dropped (flagged)
-            } else {
-                if (push) {
-                    const int j = sp + 2 * (at + __popc(m & ((1u << lane) - 1u)));
-                    stk[j] = ch.y;
-                    stk[j + 1] = ch.x;
-                }
-                sp += 2 * total;
+            if (push) {
+                const int j = sp + 2 * (at + __popc(m & ((1u << lane) - 1u)));
+                stk[j] = ch.y;
+                stk[j + 1] = ch.x;
             }
+            sp += 2 * total;
             __syncthreads();
         }
         acc += a.value();
