@@ -818,13 +818,16 @@ static gwn_status enqueue_chunk(gwn_model_s* m, const void* pts, int dtype, size
                 k_few_direct<<<(unsigned)(sms * 8), B, 0, st>>>(m->tree, ws.spos, ni, few_val, ws.st);
                 k_few_direct_sum<<<1, 32 * kFewPoints, 0, st>>>(ni, m->host.n_leaves, few_val, ws.rw);
             } else {
+                // the near band: a point on the surface has two or three pairs there, so the list takes the
+                // place of the traversal's, which holds every pair that pairs2 does
+                const int near_cap = (int)std::min<long long>(ws.pair_cap, 0x7fffffff);
                 GWN_CUDA_TRY(cudaMemsetAsync(ws.rw, 0, n * sizeof(double), st));
                 k_direct3<<<dim3(nb, slices), B, 0, st>>>(m->tree, ws.spos, ni, ws.rw, ws.st, ws.counters, ws.pairs2,
                                                           ws.slow_cap, ws.olist);
                 k_pair_eval<double><<<(unsigned)(sms * kEvalBlocks), B, 0, st>>>(m->tree, ws.spos, ws.slow_cap, ws.counters + 8,
-                                                                       ws.counters, ws.pairs2, ws.rw, ws.st, ws.pairs64, ni,
-                                                                       nullptr);
-                k_pair_eval64_warp<double><<<(unsigned)(sms * 2), B, 0, st>>>(m->tree, ws.spos, ni, ws.counters, ws.pairs64,
+                                                                       ws.counters, ws.pairs2, ws.rw, ws.st, ws.pairs,
+                                                                       near_cap, nullptr);
+                k_pair_eval64_warp<double><<<(unsigned)(sms * 2), B, 0, st>>>(m->tree, ws.spos, near_cap, ws.counters, ws.pairs,
                                                                               ws.rw, ws.st);
                 if ((long long)n * m->host.n_leaves > ws.slow_cap)
                     k_direct_overflow3<<<(unsigned)(sms * 4), B, 0, st>>>(m->tree, ws.spos, ws.rw, ws.st, ws.counters, ws.olist);

@@ -131,3 +131,19 @@ def test_fp64_sums_stay_finite_far_away():
     for mode in (gwn.MODE_BVH, gwn.MODE_DIRECT):
         w, _, _ = m.query(torch.from_numpy(q).cuda(), precision=gwn.PREC_FP64, mode=mode)
         assert float(w.abs().max()) <= 1e-15
+
+
+@pytest.mark.parametrize("n", [40, 2049, 20001])
+def test_direct_sum_on_the_surface(oracle_lib, n):
+    """Points 1e-5 off the faces have two or more near-band pairs each: the FP32 direct sum without repair
+    keeps the FP32 path's bound."""
+    patches = configs.cad_3d(seed=5, n_patches=60)[0]
+    q = _on_faces(patches, n, 11, 1e-5)
+    m = gwn.gwn_build_3d(patches, beta=6.0)
+    w, _, st = m.query(torch.from_numpy(q).cuda(), mode=gwn.MODE_DIRECT, precision=gwn.PREC_FP32)
+    bad = (st & (gwn.QS_UNRESOLVED | gwn.QS_STACK_OVERFLOW)) != 0
+    assert int(bad.sum()) <= n // 1000  # a point may lie on a trimming curve
+    idx = np.unique(np.r_[0, n - 1, np.random.default_rng(1).integers(0, n, 400)])
+    w_ref, _ = oracle_lib.gwn3d(patches, q[idx].astype(np.float64))
+    ok = np.isfinite(w_ref) & ~bad.cpu().numpy()[idx]
+    assert ok.mean() > 0.95 and np.max(np.abs(w.cpu().numpy()[idx][ok] - w_ref[ok])) <= 1e-4
