@@ -539,7 +539,10 @@ size_t workspace_layout(int dim, int n_leaves, size_t n, char* base, Workspace* 
     w.rw = (double*)carve(n * sizeof(double));
     w.rval = (double*)carve((dim != 2 ? (size_t)kRepairPairCap : 0) * sizeof(double));
     w.rcnt = (int*)carve((dim != 2 ? n : 0) * sizeof(int));
-    w.pairs64 = (int2*)carve((dim != 2 ? n : 0) * sizeof(int2));
+    // the near band: two or three pairs for a point on the surface, and whatever a small query has
+    const long long near = dim == 2 ? 0 : (long long)n * 4 + (1 << 18);
+    w.near_cap = (int)near;
+    w.pairs64 = (int2*)carve((size_t)near * sizeof(int2));
     w.rlist = (int*)carve(n * sizeof(int));
     w.rlist_g = (int*)carve(n * sizeof(int));
     w.rst = (uint32_t*)carve(n * sizeof(uint32_t));
@@ -826,7 +829,7 @@ static gwn_status enqueue_chunk(gwn_model_s* m, const void* pts, int dtype, size
                                                           ws.slow_cap, ws.olist);
                 k_pair_eval<double><<<(unsigned)(sms * kEvalBlocks), B, 0, st>>>(m->tree, ws.spos, ws.slow_cap, ws.counters + 8,
                                                                        ws.counters, ws.pairs2, ws.rw, ws.st, ws.pairs,
-                                                                       near_cap, nullptr);
+                                                                       near_cap, nullptr, nullptr);
                 k_pair_eval64_warp<double><<<(unsigned)(sms * 2), B, 0, st>>>(m->tree, ws.spos, near_cap, ws.counters, ws.pairs,
                                                                               ws.rw, ws.st);
                 if ((long long)n * m->host.n_leaves > ws.slow_cap)
@@ -857,10 +860,12 @@ static gwn_status enqueue_chunk(gwn_model_s* m, const void* pts, int dtype, size
             k_few_fast<<<(unsigned)(sms * 16), B, 0, st>>>(m->tree, ws.spos, few_cap, ws.counters, ws.pairs2, ws.wacc,
                                                            ws.st, ws.pairs, p.work);
             if (prof) GWN_CUDA_TRY(cudaEventRecord(ev[4], st));
+            // with repair a point past one near-band pair a point is evaluated whole in FP64, as always
+            const int near_cap = p.precision == GWN_PREC_FP32 ? ws.near_cap : ni;
             k_few_eval<<<(unsigned)(sms * 8), B, 0, st>>>(m->tree, ws.spos, ws.counters, ws.pairs, ws.wacc, ws.st,
-                                                          ws.pairs64, ni, p.work);
+                                                          ws.pairs64, near_cap, p.work);
             if (prof) GWN_CUDA_TRY(cudaEventRecord(ev[3], st));
-            k_pair_eval64_warp<float><<<(unsigned)(sms * 2), B, 0, st>>>(m->tree, ws.spos, ni, ws.counters, ws.pairs64,
+            k_pair_eval64_warp<float><<<(unsigned)(sms * 2), B, 0, st>>>(m->tree, ws.spos, near_cap, ws.counters, ws.pairs64,
                                                                          ws.wacc, ws.st);
             if ((long long)n * m->host.n_leaves > few_cap)
                 k_overflow3<<<1, B, 0, st>>>(m->tree, ws.spos, p.beta2, ws, ws.olist);
@@ -906,10 +911,10 @@ static gwn_status enqueue_chunk(gwn_model_s* m, const void* pts, int dtype, size
                     m->tree, ws.spos, ni, p.beta2, again ? p.beta2 : p.beta2_leaf, m->stack_depth, m->cuts[level], ws,
                     p.work, ws.olist, d, again);
             };
-            auto eval_pass = [&]() {
+            auto eval_pass = [&](int* olist) {
                 k_pair_eval<float><<<(unsigned)(sms * kEvalBlocks), B, 0, st>>>(m->tree, ws.spos, ws.slow_cap, ws.counters + 8,
-                                                               ws.counters, ws.pairs2, ws.wacc, ws.st, ws.pairs64, ni,
-                                                               p.work);
+                                                               ws.counters, ws.pairs2, ws.wacc, ws.st, ws.pairs64,
+                                                               ws.near_cap, olist, p.work);
             };
             const unsigned wide_blocks =
                 (unsigned)std::min(std::max((n + 3) / 4, std::min(n, (size_t)sms)), (size_t)sms * 16);
@@ -941,23 +946,24 @@ static gwn_status enqueue_chunk(gwn_model_s* m, const void* pts, int dtype, size
                     m->tree, ws.spos, ws.pair_cap, ws.counters, reinterpret_cast<const int4*>(ws.pairs), ws.wacc, ws.st,
                     ws.pairs2, ws.slow_cap, ws.olist, p.work);
             if (prof) GWN_CUDA_TRY(cudaEventRecord(ev[4], st));
-            eval_pass();
+            eval_pass(ws.olist);
             if (prof) GWN_CUDA_TRY(cudaEventRecord(ev[3], st));
             const bool may_overflow = (long long)n * m->host.n_leaves > ws.slow_cap;
             if (may_overflow) {
                 // the points whose pairs did not fit the list, one warp each, without a list
                 k_next_round<<<1, 32, 0, st>>>(ws);
                 wide_pass(false, (unsigned)(sms * 8), ws.olist, ws.counters + 5, dense, false);
-                eval_pass();
+                eval_pass(ws.olist2);
             }
             GWN_CUDA_TRY(cudaGetLastError());
-            // the near band of both passes in one launch: the second pass only takes
-            // points whose pairs overflowed in the first, and those have not entered
-            // the near band, so every listed point's FP32 sum is final here
-            k_pair_eval64_warp<float><<<(unsigned)(sms * 2), B, 0, st>>>(m->tree, ws.spos, ni, ws.counters, ws.pairs64,
+            // the near band of both passes in one launch: a point of the second pass has entered it
+            // only where the near band's list was full, and then it overflows in the second
+            // pass too, so every listed point's FP32 sum is final here or k_overflow3's
+            k_pair_eval64_warp<float><<<(unsigned)(sms * 2), B, 0, st>>>(m->tree, ws.spos, ws.near_cap, ws.counters, ws.pairs64,
                                                                   ws.wacc, ws.st);
-            if (may_overflow)
-                k_overflow3<<<(unsigned)(sms * 2), B, 0, st>>>(m->tree, ws.spos, p.beta2, ws, ws.olist2);
+            if (may_overflow || (long long)n * m->host.n_leaves > ws.near_cap)
+                k_overflow3<<<(unsigned)(sms * 2), B, 0, st>>>(m->tree, ws.spos, p.beta2, ws,
+                                                               may_overflow ? ws.olist2 : ws.olist);
         }
         GWN_CUDA_TRY(cudaGetLastError());
         // 4. outputs and the repair list
@@ -1546,11 +1552,12 @@ __global__ void __launch_bounds__(128) k_query_noalloc2(DevTree t, const void* p
 // 3D: one warp per point with the far exact leaves in place (k_wide3), the near ones
 // through a list, kNoAllocStep points at a time so that everything fits the
 // fixed scratch: per point 16 bytes of position, 4 + 4 + 4 + 4 of sums, status and
-// lists, 8 + 4 of FP64 sums and 8 near-band bytes, and 8 near pairs of 8 bytes
-// (points with more are evaluated by one thread, k_overflow3): 116 bytes.  100,000
+// lists, 4 of FP64 status, 8 near pairs and 3 near-band pairs of 8 bytes (points with more are
+// evaluated by one thread, k_overflow3; the repair's sums follow in the place of the third
+// near-band pair): 124 bytes.  100,000
 // points on 1.4k leaves, one thread per point with its leaves in place before: 44 ms.
 constexpr size_t kNoAllocStep = 32768;
-static_assert(kNoAllocStep * 116 + 4096 <= sizeof(int) * kNoAllocMaxPoints, "the no-alloc scratch holds one step");
+static_assert(kNoAllocStep * 124 + 4096 <= sizeof(int) * kNoAllocMaxPoints, "the no-alloc scratch holds one step");
 
 gwn_status noalloc_3d(gwn_model_s* m, const QueryParams& p, const void* points, int dtype, size_t n, double* out_w,
                       int32_t* out_label, uint32_t* out_status, int* scratch, int sms, cudaStream_t st) {
@@ -1565,16 +1572,17 @@ gwn_status noalloc_3d(gwn_model_s* m, const QueryParams& p, const void* points, 
     ws.counters = scratch;
     ws.gcount = scratch + kCounterCount;
     ws.spos = (float4*)carve(C * 16);
-    ws.rw = (double*)carve(C * 8);
     ws.pairs2 = (int2*)carve(C * 64);
     ws.slow_cap = (long long)C * 8;
-    ws.pairs64 = (int2*)carve(C * 8);
+    ws.pairs64 = (int2*)carve(C * 24);
+    ws.rw = (double*)(ws.pairs64 + 2 * C);
     ws.wacc = (float*)carve(C * 4);
     ws.st = (uint32_t*)carve(C * 4);
     ws.rst = (uint32_t*)carve(C * 4);
     ws.olist2 = (int*)carve(C * 4);
     ws.rlist_g = (int*)carve(C * 4);
     const bool o3 = m->tree.order3 != 0;
+    const int near_cap = (int)(3 * C);
     const size_t esz = (dtype == GWN_F32 ? sizeof(float) : sizeof(double)) * 3;
     const int B = 128;
     for (size_t off = 0; off < n; off += C) {
@@ -1593,9 +1601,10 @@ gwn_status noalloc_3d(gwn_model_s* m, const QueryParams& p, const void* points, 
                 m->tree, ws.spos, c, nullptr, nullptr, p.beta2, p.beta2_leaf, ws, ws.pairs2, ws.slow_cap, ws.olist2, nullptr,
                 Dense{nullptr, 0}, false);
         k_pair_eval<float><<<(unsigned)(sms * kEvalBlocks), B, 0, st>>>(m->tree, ws.spos, ws.slow_cap, ws.counters + 8, ws.counters,
-                                                              ws.pairs2, ws.wacc, ws.st, ws.pairs64, c, nullptr);
-        k_pair_eval64_warp<float><<<(unsigned)(sms * 2), B, 0, st>>>(m->tree, ws.spos, c, ws.counters, ws.pairs64, ws.wacc,
-                                                                     ws.st);
+                                                              ws.pairs2, ws.wacc, ws.st, ws.pairs64, near_cap,
+                                                              ws.olist2, nullptr);
+        k_pair_eval64_warp<float><<<(unsigned)(sms * 2), B, 0, st>>>(m->tree, ws.spos, near_cap, ws.counters, ws.pairs64,
+                                                                     ws.wacc, ws.st);
         k_overflow3<<<(unsigned)(sms * 2), B, 0, st>>>(m->tree, ws.spos, p.beta2, ws, ws.olist2);
         k_finish<float><<<nb, B, 0, st>>>(c, ws.spos, ws.wacc, ws.st, p.precision, p.band, w, label, status, nullptr, nullptr,
                                           0, ws.rlist_g, ws.gcount, c);

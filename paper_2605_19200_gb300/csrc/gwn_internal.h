@@ -258,7 +258,8 @@ struct RepairList {
 // Scratch of one in-flight query (one chunk of points), carved from one
 // device allocation (see workspace_layout in gwn_api.cu).
 struct Workspace {
-    int2* pairs64;    // near-band pairs (capacity n)
+    int2* pairs64;    // near-band pairs (near_cap)
+    int near_cap;
     int2* rpairs;     // FP64 repair pairs (kRepairPairCap, 3D)
     int2* rpairs2;    // of which the full FP64 evaluator takes (kRepairPairCap, 3D)
     double* rw;       // FP64 repair accumulators (n)

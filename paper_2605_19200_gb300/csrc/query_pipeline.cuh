@@ -1096,15 +1096,16 @@ __global__ void __launch_bounds__(128) k_direct_overflow3(DevTree t, const float
 //   4. rounds over the listed panels, four lanes to a panel (one Gauss-Legendre node
 //      each, from the curve's Bernstein form): the integral, or two panels of
 //      the next level for the next round.
-// Pairs FP32 cannot resolve go to the FP64 near band.  One thread doing all of this for
-// its pair from the Bernstein form alone (28 D + 70 flops per node, the tables 34) took
+// Pairs FP32 cannot resolve go to the FP64 near band; where its list is full their point goes
+// to olist (the points evaluated again in place), or, without one, is flagged for the repair.
+// One thread doing all of this for its pair from the Bernstein form alone (28 D + 70 flops per node, the tables 34) took
 // 5.8 ms on 1.3M points of a 4.7k-leaf model, whole curves below level 1 per
 // thread 1.8 ms with 10 to 12 active lanes per instruction.
 constexpr int kNearHalves = 2048, kNearPanels = 1024;
 template <typename Acc>  // float, or double (the direct sum)
 __global__ void __launch_bounds__(128, 5) k_pair_eval(DevTree t, const float4* spos, long long npair_cap,
                                                    const int* count, int* counters, const int2* pairs, Acc* wacc,
-                                                   uint32_t* st, int2* pairs64, int npair64_cap,
+                                                   uint32_t* st, int2* pairs64, int npair64_cap, int* olist,
                                                    unsigned long long* work) {
     __shared__ float sq[3][128], ss[3][128], sacc[128];
     __shared__ int sleaf[128], sfail[128], shit[128];
@@ -1300,8 +1301,14 @@ __global__ void __launch_bounds__(128, 5) k_pair_eval(DevTree t, const float4* s
                 atomicAdd(&wacc[pr.x], (Acc)sacc[tid]);
             } else {
                 const int slot = atomicAdd(&counters[2], 1);
-                if (slot < npair64_cap) pairs64[slot] = pr;
-                atomicOr(&st[pr.x], slot < npair64_cap ? GWN_QS_NEAR : GWN_QS_STACK_OVERFLOW);
+                if (slot < npair64_cap) {
+                    pairs64[slot] = pr;
+                    atomicOr(&st[pr.x], GWN_QS_NEAR);
+                } else if (!olist) {
+                    atomicOr(&st[pr.x], GWN_QS_STACK_OVERFLOW);
+                } else if (!(atomicOr(&st[pr.x], kPairOverflow) & kPairOverflow)) {
+                    olist[atomicAdd(&counters[3], 1)] = pr.x;
+                }
             }
         }
         __syncthreads();  // the lists are reset next
@@ -1332,6 +1339,7 @@ __global__ void __launch_bounds__(128) k_pair_eval64_warp(DevTree t, const float
     // few pairs: an SM each first, since the warps of an SM share its two FP64 lanes
     for (int k = wid * gridDim.x + blockIdx.x; k < np; k += gridDim.x * 4) {
         const int2 pr = pairs64[k];
+        if (st[pr.x] & kPairOverflow) continue;  // evaluated again in place
         const float4 p = spos[pr.x];
         const double q[3] = {(double)p.x, (double)p.y, (double)p.z};
         double v = 0;

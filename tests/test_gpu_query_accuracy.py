@@ -147,3 +147,23 @@ def test_direct_sum_on_the_surface(oracle_lib, n):
     w_ref, _ = oracle_lib.gwn3d(patches, q[idx].astype(np.float64))
     ok = np.isfinite(w_ref) & ~bad.cpu().numpy()[idx]
     assert ok.mean() > 0.95 and np.max(np.abs(w.cpu().numpy()[idx][ok] - w_ref[ok])) <= 1e-4
+
+
+@pytest.mark.parametrize("n", [3, 40, 5000, 40000])
+def test_near_band_on_the_surface(oracle_lib, n):
+    """Points 1e-5 off the faces have two or more near-band pairs each: the traversal without repair and the
+    no-alloc call evaluate them all (flagged where a list is full), within the FP32 path's bound."""
+    patches = configs.cad_3d(seed=5, n_patches=60)[0]
+    q = _on_faces(patches, n, 12, 1e-5)
+    m = gwn.gwn_build_3d(patches, beta=6.0, beta_leaf=4.0)
+    pts = torch.from_numpy(q).cuda()
+    out = (torch.empty(n, dtype=torch.float64, device="cuda"), torch.empty(n, dtype=torch.int32, device="cuda"),
+           torch.empty(n, dtype=torch.int32, device="cuda"))
+    idx = np.unique(np.r_[0, n - 1, np.random.default_rng(1).integers(0, n, 400)])
+    w_ref, _ = oracle_lib.gwn3d(patches, q[idx].astype(np.float64))
+    ok = np.isfinite(w_ref)
+    assert ok.mean() > 0.95
+    for w, _, st in (m.query(pts, precision=gwn.PREC_FP32), gwn.api.gwn_query_noalloc(m, pts, out)):
+        assert int(((st & gwn.QS_STACK_OVERFLOW) != 0).sum()) == 0
+        good = ok & ((st & gwn.QS_UNRESOLVED) == 0).cpu().numpy()[idx]
+        assert np.max(np.abs(w.cpu().numpy()[idx][good] - w_ref[good])) <= 1e-4
