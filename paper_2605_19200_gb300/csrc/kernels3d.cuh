@@ -835,61 +835,11 @@ __device__ inline void net_eval3_warp(const G& g, T u, T v, T S[3], T Su[3], T S
     }
 }
 
-// curve_angle in FP32 for decisions that FP64 would take alike: a box that holds the origin
-// within a margin well above FP32 rounding counts as holding it, and a curve that
-// needs more than kNear32 levels is left to FP64 (false)
-__device__ inline bool curve_angle32_sure(const double (&Hd)[4][3], float* out) {
-    float H[4][3], m = 0.f;
-    for (int i = 0; i < 4; ++i)
-        for (int k = 0; k < 3; ++k) {
-            H[i][k] = (float)Hd[i][k];
-            if (k < 2) m = fmaxf(m, fabsf(H[i][k]) / H[i][2]);
-        }
-    const float eps = 4e-6f * m;  // control points are rounded to 6e-8 m, the splits to a few times that
-    float acc = 0;
-    int level = 0;
-    unsigned idx = 0;
-    while (true) {
-        float h[4][3];
-        for (int i = 0; i < 4; ++i)
-            for (int k = 0; k < 3; ++k) h[i][k] = H[i][k];
-        if (level > 0) {
-            const float sc = 1.f / (float)(1u << level), t0 = (float)idx * sc, t1 = (float)(idx + 1) * sc;
-            if (t1 < 1.f) cubic_part(h, t1, true);
-            if (t0 > 0.f) cubic_part(h, t0 / t1, false);
-        }
-        float ex[4], ey[4];
-        for (int i = 0; i < 4; ++i) {
-            const float iw = __fdividef(1.f, h[i][2]);
-            ex[i] = h[i][0] * iw;
-            ey[i] = h[i][1] * iw;
-        }
-        const float lx = fminf(fminf(ex[0], ex[1]), fminf(ex[2], ex[3])), hx = fmaxf(fmaxf(ex[0], ex[1]), fmaxf(ex[2], ex[3]));
-        const float ly = fminf(fminf(ey[0], ey[1]), fminf(ey[2], ey[3])), hy = fmaxf(fmaxf(ey[0], ey[1]), fmaxf(ey[2], ey[3]));
-        if (!(lx > eps || hx < -eps || ly > eps || hy < -eps)) {
-            if (level == kNear32) return false;
-            ++level;
-            idx <<= 1;
-            continue;
-        }
-        acc += atan2f(ex[0] * ey[3] - ey[0] * ex[3], ex[0] * ex[3] + ey[0] * ey[3]);
-        while (idx & 1u) {
-            idx >>= 1;
-            --level;
-        }
-        if (level == 0) break;
-        ++idx;
-    }
-    *out = acc;
-    return true;
-}
-
-// curve_angle<double> for a winding number: the same pieces are split off in FP64, but the
-// box tests look at the signs of the homogeneous coordinates (the weights are positive)
-// and the pieces' angles, of which only the integer sum counts, come from FP32: about
-// 80 FP64 instructions a piece instead of 240
-__device__ inline bool curve_angle_signs64(const double (&H)[4][3], int maxlevel, float* out) {
-    float acc = 0;
+// curve_angle<double> for a winding number: the same pieces, but the box tests look at the
+// signs of the homogeneous coordinates (the weights are positive) and the chord angles are those
+// of the homogeneous end points, so that a piece needs no division
+__device__ inline bool curve_angle_signs64(const double (&H)[4][3], int maxlevel, double* out) {
+    double acc = 0;
     int level = 0;
     unsigned long long idx = 0;
     bool ok = true;
@@ -917,7 +867,7 @@ __device__ inline bool curve_angle_signs64(const double (&H)[4][3], int maxlevel
             continue;
         }
         if (inside) ok = false;
-        acc += atan2f((float)(h[0][0] * h[3][1] - h[0][1] * h[3][0]), (float)(h[0][0] * h[3][0] + h[0][1] * h[3][1]));
+        acc += atan2(h[0][0] * h[3][1] - h[0][1] * h[3][0], h[0][0] * h[3][0] + h[0][1] * h[3][1]);
         while (idx & 1ull) {
             idx >>= 1;
             --level;
@@ -933,33 +883,23 @@ __device__ inline bool curve_angle_signs64(const double (&H)[4][3], int maxlevel
 // (on: this lane has one); false if a curve comes too close to the origin to decide
 __device__ inline bool winding_warp(bool on, const double (&H)[4][3], double m, int* wind) {
     const unsigned full = 0xffffffffu;
-    float a32 = 0.f;
-    const bool sure = !on || curve_angle32_sure(H, &a32);
-    if (__all_sync(full, sure)) {
-        a32 *= (float)m;
-        for (int off = 16; off > 0; off >>= 1) a32 += __shfl_xor_sync(full, a32, off);
-        const float w = a32 * Num<float>::inv2pi;
-        *wind = (int)roundf(w);
-        if (fabsf(w - roundf(w)) < 0.01f) return true;
-    }
-    bool ok = true;
-    a32 = 0.f;
-    if (on) ok = curve_angle_signs64(H, kMaxLevel64, &a32);
+    double a = 0;
+    const bool ok = !on || curve_angle_signs64(H, kMaxLevel64, &a);
     if (!__all_sync(full, ok)) return false;
-    a32 *= (float)m;
-    for (int off = 16; off > 0; off >>= 1) a32 += __shfl_xor_sync(full, a32, off);
-    if (a32 != a32) return false;  // a NaN coordinate
-    *wind = (int)roundf(a32 * Num<float>::inv2pi);
+    a *= m;
+    for (int off = 16; off > 0; off >>= 1) a += __shfl_xor_sync(full, a, off);
+    if (a != a) return false;  // a NaN coordinate
+    *wind = (int)round(a * Num<double>::inv2pi);
     return true;
 }
 
 // leaf_hit in FP64 with a warp for one point: the rejects from the leaf's FP32 bounds
 // (conservative, t.lhit), the windings of the four edge curves and then of the trim
-// curves one curve per lane, in FP32 where that decides them (integers), and the foot
-// point from an FP32 solution, which leaves two or three FP64 steps.  In one lane
-// all of it ran at FP64 latency -- every instruction holds the FP64 pipe for a
-// warp's time whatever the active lanes -- and a single near-band pair took 260 us of a
-// 1.5 ms query; with the windings in FP64 over the lanes 190 us.
+// curves one curve per lane, and the foot point from an FP32 solution, which leaves two or three
+// FP64 steps.  In one lane all of it ran at FP64 latency -- every instruction holds the
+// FP64 pipe for a warp's time whatever the active lanes -- and a single near-band pair took
+// 260 us of a 1.5 ms query.  (Windings from FP32 pieces where a margin allows were 50 to 70 us
+// shorter, and are not taken: this is the FP64 evaluation.)
 __device__ inline int leaf_hit64_warp(const DevTree& t, int li, const Leaf3Info& I, const Geo64& g, const double q[3],
                                       const double nrm[3], double sig, double* contrib) {
     const unsigned full = 0xffffffffu;
