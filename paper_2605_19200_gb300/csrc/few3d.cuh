@@ -43,6 +43,7 @@ __global__ void __launch_bounds__(32) k_few_walk(DevTree t, const float4* spos, 
     float w = 0.f;
     uint32_t st = 0;
     int bcnt = 0;      // warp-uniform: entries in buf
+    unsigned nfound = 0;
     unsigned ovf = 0;  // lanes with pairs that did not fit the list
     int sp = 0;        // warp-uniform
 
@@ -72,6 +73,7 @@ __global__ void __launch_bounds__(32) k_few_walk(DevTree t, const float4* spos, 
                     buf[pos] = make_int2(qi, li);
                     own[pos] = (unsigned char)lane;
                 }
+                nfound += nn;
                 bcnt += nn;
             }
             return 0u;
@@ -126,6 +128,7 @@ __global__ void __launch_bounds__(32) k_few_walk(DevTree t, const float4* spos, 
         ws.st[qi] = st;
         if (st & kPairOverflow) olist_out[atomicAdd(&ws.counters[3], 1)] = qi;
     }
+    if (lane == 0 && nfound) atomicAdd(ws.found, (unsigned long long)nfound);
     if (work) flush_work(wl, work);
 }
 

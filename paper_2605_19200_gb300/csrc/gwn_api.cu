@@ -553,7 +553,7 @@ size_t workspace_layout(int dim, int n_leaves, size_t n, char* base, Workspace* 
     // control words, 256 bytes each, cleared together: the query's, then the chunk's
     w.acc = (unsigned long long*)carve(kCounterCount * sizeof(unsigned long long));
     w.gcount = (int*)carve(8 * sizeof(int));
-    w.counters = (int*)carve(kCounterCount * sizeof(int) + sizeof(unsigned long long));
+    w.counters = (int*)carve(kCounterCount * sizeof(int) + 2 * sizeof(unsigned long long));
     w.found = (unsigned long long*)(w.counters + kCounterCount);  // cleared with the counters
     w.bbox = (unsigned*)carve(8 * sizeof(unsigned));
     w.pair_cap = cap;
@@ -1571,6 +1571,7 @@ gwn_status noalloc_3d(gwn_model_s* m, const QueryParams& p, const void* points, 
     Workspace ws{};
     ws.counters = scratch;
     ws.gcount = scratch + kCounterCount;
+    ws.found = (unsigned long long*)(scratch + 2 * kCounterCount);
     ws.spos = (float4*)carve(C * 16);
     ws.pairs2 = (int2*)carve(C * 64);
     ws.slow_cap = (long long)C * 8;
@@ -1675,7 +1676,6 @@ gwn_status gwn_last_query_stats(gwn_model m, int64_t* out) {
     }
     for (int k = 0; k < kQueryStats; ++k) out[k] = 0;
     for (int k = 0; k < 4; ++k) out[k] = (int64_t)c[k];
-    out[0] = (int64_t)(c[0] + c[7] - c[11]);  // pairs of both passes, without the padding
     out[2] = (int64_t)c[2];           // near-band (FP64) pairs over all rounds
     out[3] = (int64_t)(c[6] + c[3]);  // points whose pairs overflowed in any round
     for (int k = 0; k < 8; ++k) out[4 + k] = (int64_t)wk[k];

@@ -275,12 +275,12 @@ struct Workspace {
     int2* pairs;      // pair capacity: (point, leaf) pairs of the traversal, in runs of one leaf (k_trav3: of
                       // even length, padded with point -1)
     int2* pairs2;     // slow capacity: those the node tables left to the full evaluator
-    int* counters;    // [0] pairs, [1] repair count, [2] near-band pairs, [3] overflowed points, [4] repair pairs,
+    int* counters;    // [0] entries of the pair list, [1] repair count, [2] near-band pairs, [3] overflowed points, [4] repair pairs,
                       // [5] overflowed points of the first pass (list input of the second), [6] total overflow,
-                      // [7] pairs of the first pass, [8] pairs left to the full evaluator in this pass,
-                      // [9] the same in the first pass, [10] repair pairs the FP64 tables left,
-                      // [11] padding entries of the pair list
-    unsigned long long* found;  // (point, leaf) pairs that the chunk's first walk needs exactly, listed or not
+                      // [8] pairs left to the full evaluator in this pass,
+                      // [9] the same in the first pass, [10] repair pairs the FP64 tables left
+    unsigned long long* found;  // (point, leaf) pairs needed exactly, listed or not: [0] of the chunk's first walk,
+                                // [1] of the later ones
     int* olist;       // n: points whose pairs did not fit in the first pass
     int* olist2;      // n: in the second
     unsigned long long* work;  // kWorkCount counters

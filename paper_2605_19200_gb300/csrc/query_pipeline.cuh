@@ -278,7 +278,7 @@ __global__ void k_dense_reset(Workspace ws, int n, Dense d) {
         ws.wacc[i] = 0.f;
         ws.st[i] = 0u;
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) ws.counters[0] = ws.counters[3] = ws.counters[11] = 0;
+    if (blockIdx.x == 0 && threadIdx.x == 0) ws.counters[0] = ws.counters[3] = 0;
 }
 
 // bytes of dynamic shared memory of k_trav3 (one warp) with a stack of `depth` entries
@@ -344,7 +344,7 @@ __global__ void __launch_bounds__(32, 28) k_trav3(DevTree t, const float4* spos,
     }
     float w0 = 0.f, w1 = 0.f;
     uint32_t st0 = 0, st1 = 0;
-    int bcnt = 0, npad = 0;            // warp-uniform: entries in buf, padding entries so far
+    int bcnt = 0;                      // warp-uniform: entries in buf
     unsigned nfound = 0;               // warp-uniform: exact pairs
     unsigned ovf0 = 0, ovf1 = 0;       // queries with pairs that did not fit the list
     int sp = 0;                        // warp-uniform
@@ -397,7 +397,6 @@ __global__ void __launch_bounds__(32, 28) k_trav3(DevTree t, const float4* spos,
                     buf[bcnt + nn] = make_int2(-1, ~c);
                     own[bcnt + nn] = 64;
                 }
-                npad += even - nn;
                 nfound += nn;
                 bcnt += even;
             }
@@ -453,8 +452,7 @@ __global__ void __launch_bounds__(32, 28) k_trav3(DevTree t, const float4* spos,
     }
     __syncwarp();
     flush_packet_pairs(buf, own, bcnt, ws, ovf0, ovf1);
-    if (lane == 0 && npad) atomicAdd(&ws.counters[11], npad);
-    if (lane == 0 && nfound && !again) atomicAdd(ws.found, (unsigned long long)nfound);
+    if (lane == 0 && nfound) atomicAdd(ws.found + again, (unsigned long long)nfound);
     if (ovf0 & lbit) st0 |= kPairOverflow;
     if (ovf1 & lbit) st1 |= kPairOverflow;
     auto put = [&](int q, float w, uint32_t st) {
@@ -709,7 +707,7 @@ __global__ void __launch_bounds__(128) k_wide3(DevTree t, const float4* spos, in
     if (n_dev) n = *n_dev;
     const float b2l = t.leaf_far ? (is_dense(d) ? beta2 : beta2l) : INFINITY;
     const float ratio2 = kRatio32 * kRatio32, inv4pi = 0.07957747154594767f;
-    int npair = 0;
+    unsigned long long npair = 0;
     // few points: a block (an SM) each first
     for (int k = wid * gridDim.x + blockIdx.x; k < n; k += gridDim.x * 4) {
         const int qi = list ? list[k] : k;
@@ -737,8 +735,8 @@ __global__ void __launch_bounds__(128) k_wide3(DevTree t, const float4* spos, in
             __syncwarp();
         };
         auto exact_leaves = [&]() {
+            npair += nl;
             if (LIST) {
-                npair += nl;
                 long long base = 0;
                 if (lane == 0 && nl) base = list_slots(&ws.counters[0], nl, ws.pair_cap);
                 base = __shfl_sync(full, base, 0);
@@ -804,7 +802,6 @@ __global__ void __launch_bounds__(128) k_wide3(DevTree t, const float4* spos, in
                     if (__shfl_sync(full, slot, 0) >= slow_cap) st |= kPairOverflow;
                 }
             }
-            npair += nl;
             nl = 0;
             __syncwarp();
         };
@@ -852,8 +849,7 @@ __global__ void __launch_bounds__(128) k_wide3(DevTree t, const float4* spos, in
         }
         __syncwarp();
     }
-    if (!LIST && lane == 0 && npair) atomicAdd(&ws.counters[0], npair);
-    if (LIST && !again && lane == 0 && npair) atomicAdd(ws.found, (unsigned long long)npair);
+    if (lane == 0 && npair) atomicAdd(ws.found + (!LIST || again), npair);
     if (COUNT) flush_work(wl, work);
 }
 
@@ -1489,7 +1485,6 @@ __global__ void k_next_round(Workspace ws) {
     if (threadIdx.x == 0) {
         ws.counters[5] = ws.counters[3];
         ws.counters[6] += ws.counters[3];
-        ws.counters[7] += ws.counters[0];  // pairs of the finished round
         ws.counters[9] += ws.counters[8];  // of which the full evaluator took
         ws.counters[3] = 0;
         ws.counters[0] = 0;  // the near-band list (counters[2]) spans all rounds
@@ -1501,7 +1496,7 @@ __global__ void k_next_round(Workspace ws) {
 // (repaired points and FP64 pairs)
 __global__ void k_accum(Workspace ws, bool last) {
     const int k = threadIdx.x;
-    if (k < kCounterCount) ws.acc[k] += (unsigned long long)ws.counters[k];
+    if (k < kCounterCount) ws.acc[k] += k == 0 ? ws.found[0] + ws.found[1] : (unsigned long long)ws.counters[k];
     if (!last) return;
     __syncwarp();
     if (k == 0) ws.acc[1] += (unsigned long long)min(ws.gcount[0], ws.rcap);

@@ -167,3 +167,20 @@ def test_near_band_on_the_surface(oracle_lib, n):
         assert int(((st & gwn.QS_STACK_OVERFLOW) != 0).sum()) == 0
         good = ok & ((st & gwn.QS_UNRESOLVED) == 0).cpu().numpy()[idx]
         assert np.max(np.abs(w.cpu().numpy()[idx][good] - w_ref[good])) <= 1e-4
+
+
+@pytest.mark.parametrize("n,side", [(5, 6), (4000, 6), (5003, 6), (290001, 20), (1 << 20, 64)])
+def test_pair_count(n, side):
+    """Every leaf exact for every point: the statistics count n pairs a leaf, and those of the points that
+    are evaluated again, without the list's padding and beyond 2^32."""
+    from synth import geometry as G
+    patches = [G.planar_patch((i, j, 0), (0.9, 0, 0), (0, 0.9, 0)) for i in range(side) for j in range(side)]
+    m = gwn.gwn_build_3d(patches, max_aabb_frac=0.0, beta=1e4, beta_leaf=1e4, precision=gwn.PREC_FP32)
+    nl = m.info()["n_leaves"]
+    g = torch.Generator(device="cuda").manual_seed(1)
+    q = torch.rand(n, 3, generator=g, device="cuda") * torch.tensor([side, side, 1.0], device="cuda")
+    q[:, 2] += 2.0
+    m.query(q)
+    s = m.last_query_stats()
+    assert s["pairs"] == nl * (n + s["overflow"])
+    assert n < (1 << 20) or s["pairs"] > 2 ** 32
