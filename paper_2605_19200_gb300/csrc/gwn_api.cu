@@ -507,11 +507,15 @@ __global__ void __launch_bounds__(128) k_repair2(DevTree t, const void* pts, int
 // Bytes of the query workspace for n points of model m, and its layout.
 // dim 0 lays out a workspace that serves both 2D and 3D models.
 size_t workspace_layout(int dim, int n_leaves, size_t n, char* base, Workspace* ws) {
-    // (point, leaf) pairs: 128 per point, and for fewer points, next to the surface of a
-    // dense model above all, up to every leaf for every point within 2^26 pairs (0.5 GB)
-    const long long cap = dim == 2 ? 0
-                                   : std::max((long long)n * 128 + 65536,
-                                              dim == 3 ? std::min((long long)n * n_leaves, 1ll << 26) & ~1ll : 0ll);
+    // (point, leaf) pairs: 128 per point, and for fewer points, which may all lie next to the
+    // surface of a dense model, up to 768 within 2^26 pairs (0.5 GB; points past it are walked
+    // again without the list); at least as many as hold the FP64 pairs' values (rval) in the place
+    // of this list and the next, which GWN_PREC_FP64 does not use
+    long long cap = 0;
+    if (dim != 2) {
+        cap = std::max((long long)n * 128 + 65536, (kRepairPairCap * 4 / 5 + 63) & ~63ll);
+        if (dim == 3) cap = std::max(cap, std::min((long long)n * std::min(n_leaves, 768), 1ll << 26) & ~63ll);
+    }
     const size_t cells = kMaxBinCells;  // the finest binning of either dimension
     const size_t hist = std::max(cells + kMaxBinCells / kScanTile,  // and the scan's tile sums
                                  (size_t)n_leaves);                // k_few_sort: an entry per leaf
@@ -537,7 +541,7 @@ size_t workspace_layout(int dim, int n_leaves, size_t n, char* base, Workspace* 
     w.part = (float*)carve((dim != 3 ? kParts2 : 0) * sizeof(float));
     w.near = (long long*)carve((dim != 3 ? n : 0) * sizeof(long long));
     w.rw = (double*)carve(n * sizeof(double));
-    w.rval = (double*)carve((dim != 2 ? (size_t)kRepairPairCap : 0) * sizeof(double));
+    w.rval = (double*)w.pairs;
     w.rcnt = (int*)carve((dim != 2 ? n : 0) * sizeof(int));
     // the near band: two or three pairs for a point on the surface, and whatever a small query has
     const long long near = dim == 2 ? 0 : (long long)n * 4 + (1 << 18);

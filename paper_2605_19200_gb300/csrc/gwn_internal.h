@@ -263,7 +263,7 @@ struct Workspace {
     int2* rpairs;     // FP64 repair pairs (kRepairPairCap, 3D)
     int2* rpairs2;    // of which the full FP64 evaluator takes (kRepairPairCap, 3D)
     double* rw;       // FP64 repair accumulators (n)
-    double* rval;     // values of the FP64 pairs (kRepairPairCap, 3D)
+    double* rval;     // values of the FP64 pairs (kRepairPairCap, 3D), in the place of pairs and pairs2
     int* rcnt;        // pairs per point (n)
     float4* spos;     // n: the chunk's points in binned order, w = index of the point in the chunk
     int* key;         // n: Morton cell of each point (binning)

@@ -184,3 +184,20 @@ def test_pair_count(n, side):
     s = m.last_query_stats()
     assert s["pairs"] == nl * (n + s["overflow"])
     assert n < (1 << 20) or s["pairs"] > 2 ** 32
+
+
+def test_small_queries_keep_a_small_workspace():
+    """A 64-point query of a model of 14,400 leaves: the FP64 repair's two pair lists (67 MB) and the
+    FP32 lists (4 million pairs, 34 MB) are most of its scratch, not a list of every leaf for every point."""
+    from synth import geometry as G
+    patches = [G.planar_patch((i, j, 0), (0.9, 0, 0), (0, 0.9, 0)) for i in range(120) for j in range(120)]
+    m = gwn.gwn_build_3d(patches, max_aabb_frac=0.0, beta=6.0, beta_leaf=4.0)
+    q = torch.rand(64, 3, device="cuda")
+    out = (torch.empty(64, dtype=torch.float64, device="cuda"), None, None)
+    small = gwn.gwn_build_3d(patches[:40], max_aabb_frac=0.0, beta=6.0, beta_leaf=4.0)
+    gwn.gwn_query(small, q, out=out)  # loads the kernels
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    gwn.gwn_query(m, q, out=out)
+    torch.cuda.synchronize()
+    assert before - torch.cuda.mem_get_info()[0] <= 128 << 20
