@@ -609,15 +609,43 @@ def main():
     if rank == 0 and world == 1 and not args.no_serve:
         serving = serving_leg(gwn, args.serve_seconds, log)
 
-    # kernels per piece of up to 2^20 points: box, bin, scan (and its tile sums above 4096 cells), scatter;
-    # traversal, node-table pairs, full pairs; the points whose pairs did not fit (switch, traversal, full
-    # pairs); near band, overflow, finish; FP64 repair x5 and the counters' sum
-    def launches(n, ppc):
-        bits = min(6, max(3, round(math.log2(max(1.0, n / ppc)) / 3)))
-        return 19 + (1 if 3 * bits > 12 else 0)
+    # kernels of one query of n points of a model, in chunks of up to 2^20 (the batch enqueues a longer
+    # item's pieces as queries of their own)
+    def launches(n, m):
+        info = m.info()
+        nl, rcap = info["n_leaves"], 1 << 20 if batch is not None else min(max(n, 4096), 1 << 20)
+        slow, near = (rcap * 128 + 65536) // 4, rcap * 4 + (1 << 18)
+        total = 0
+        for o in range(0, n, 1 << 20):
+            c = min(1 << 20, n - o)
+            over = c * nl > slow
+            limit = (96 * rcap + 65536) * min(3.3, max(1.4, 1.4 + (c - 150000) / 300000))
+            if n <= 16:      # copy; walk, sort, table pairs, full pairs
+                total += 5 + (1 if over else 0)
+            else:
+                if c <= 4096:    # copy
+                    total += 1
+                else:            # box, bin, scan (and its tile sums above 4096 cells), copy in binned order
+                    bits = min(6, max(3, round(math.log2(max(1.0, c / info["bin_points_per_cell"])) / 3)))
+                    total += 4 + (1 if 3 * bits > 12 else 0)
+                total += 3       # walk, table pairs, full pairs
+                if info["beta_leaf"] < info["beta"] and c * nl > limit:
+                    total += 2   # the second walk of a dense chunk
+                if over:
+                    total += 3   # points whose pairs did not fit: switch, walk, full pairs
+                total += 1 if over or c * nl > near else 0  # in place
+            total += 3           # near band, outputs, the counters' sum
+            if n > rcap:
+                total += repair(rcap, nl)
+        return total + repair(rcap, nl)
 
-    pieces = [(min(1 << 20, p.shape[0] - o), m) for p, m in zip(points, models) for o in range(0, p.shape[0], 1 << 20)]
-    launches_per_step = sum(launches(n, m.info()["bin_points_per_cell"]) for n, m in pieces)
+    def repair(rcap, nl):        # walk, table pairs, full pairs, marked points, outputs
+        return 5 if rcap * nl > 1 << 22 else 4
+
+    sizes = [(p.shape[0], m) for p, m in zip(points, models)]
+    if batch is not None:
+        sizes = [(min(1 << 20, n - o), m) for n, m in sizes for o in range(0, n, 1 << 20)]
+    launches_per_step = sum(launches(n, m) for n, m in sizes)
     line = {
         "metric": "GWN queries/s (batched containment, 16 trimmed-NURBS models)",
         "value": value, "unit": "queries/s", "n_gpus": world, "steps": args.steps, "warmup": max(3, args.warmup),
