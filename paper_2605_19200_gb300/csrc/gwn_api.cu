@@ -814,34 +814,40 @@ static gwn_status enqueue_chunk(gwn_model_s* m, const void* pts, int dtype, size
             key = ws.key;
         }
         if (m->dim == 2) k_scatter_points<2><<<nb, B, 0, st>>>(pts, dtype, ni, key, ws.hist, ws.spos, ws.wacc, ws.st, ws.near);
-        else k_scatter_points<3><<<nb, B, 0, st>>>(pts, dtype, ni, key, ws.hist, ws.spos, ws.wacc, ws.st, ws.near);
+        else k_scatter_points<3><<<nb, B, 0, st>>>(pts, dtype, ni, key, ws.hist, ws.spos, ws.wacc, ws.st, nullptr);
         GWN_CUDA_TRY(cudaGetLastError());
         if (direct3) {
             // every leaf for every point, the leaves in slices until the blocks fill the GPU
             const unsigned slices = (unsigned)std::max<long long>(
                 1, std::min<long long>(std::min<long long>(m->host.n_leaves, 65535), ((long long)sms * 16 + nb - 1) / nb));
             float* few_val = reinterpret_cast<float*>(ws.rpairs);  // the repair's pairs come later
+            // every point to repair goes to the chunk's own list (repaired by the direct sum below)
+            auto finish = [&](auto* acc, const long long* near) {
+                k_finish<<<nb, B, 0, st>>>(ni, ws.spos, acc, ws.st, p.precision, p.band, out_w, out_label, out_status, ws.rlist,
+                                           rcount, (int)off, ws.rlist_g, ws.gcount, 0, 0, near);
+            };
             if (few && (long long)n * m->host.n_leaves <= 2 * kRepairPairCap) {
                 k_few_direct<<<(unsigned)(sms * 8), B, 0, st>>>(m->tree, ws.spos, ni, few_val, ws.st);
                 k_few_direct_sum<<<1, 32 * kFewPoints, 0, st>>>(ni, m->host.n_leaves, few_val, ws.rw);
+                finish(ws.rw, nullptr);
             } else {
                 // the near band: a point on the surface has two or three pairs there, so the list takes the
                 // place of the traversal's, which holds every pair that pairs2 does
                 const int near_cap = (int)std::min<long long>(ws.pair_cap, 0x7fffffff);
-                GWN_CUDA_TRY(cudaMemsetAsync(ws.rw, 0, n * sizeof(double), st));
-                k_direct3<<<dim3(nb, slices), B, 0, st>>>(m->tree, ws.spos, ni, ws.rw, ws.st, ws.counters, ws.pairs2,
+                long long* acc = reinterpret_cast<long long*>(ws.rw);
+                GWN_CUDA_TRY(cudaMemsetAsync(acc, 0, n * sizeof(long long), st));
+                k_direct3<<<dim3(nb, slices), B, 0, st>>>(m->tree, ws.spos, ni, acc, ws.wacc, ws.st, ws.counters, ws.pairs2,
                                                           ws.slow_cap, ws.olist);
-                k_pair_eval<double><<<(unsigned)(sms * kEvalBlocks), B, 0, st>>>(m->tree, ws.spos, ws.slow_cap, ws.counters + 8,
-                                                                       ws.counters, ws.pairs2, ws.rw, ws.st, ws.pairs,
-                                                                       near_cap, nullptr, nullptr);
-                k_pair_eval64_warp<double><<<(unsigned)(sms * 2), B, 0, st>>>(m->tree, ws.spos, near_cap, ws.counters, ws.pairs,
-                                                                              ws.rw, ws.st);
+                k_pair_eval<long long><<<(unsigned)(sms * kEvalBlocks), B, 0, st>>>(
+                    m->tree, ws.spos, ws.slow_cap, ws.counters + 8, ws.counters, ws.pairs2, acc, ws.st, ws.pairs, near_cap,
+                    nullptr, nullptr);
+                k_pair_eval64_warp<<<(unsigned)(sms * 2), B, 0, st>>>(m->tree, ws.spos, near_cap, ws.counters, ws.pairs,
+                                                                      ws.wacc, ws.st, acc);
                 if ((long long)n * m->host.n_leaves > ws.slow_cap)
-                    k_direct_overflow3<<<(unsigned)(sms * 4), B, 0, st>>>(m->tree, ws.spos, ws.rw, ws.st, ws.counters, ws.olist);
+                    k_direct_overflow3<<<(unsigned)(sms * 4), B, 0, st>>>(m->tree, ws.spos, acc, ws.wacc, ws.st, ws.counters,
+                                                                          ws.olist);
+                finish(ws.wacc, acc);
             }
-            // every point to repair goes to the chunk's own list (repaired by the direct sum below)
-            k_finish<double><<<nb, B, 0, st>>>(ni, ws.spos, ws.rw, ws.st, p.precision, p.band, out_w, out_label, out_status,
-                                               ws.rlist, rcount, (int)off, ws.rlist_g, ws.gcount, 0);
             GWN_CUDA_TRY(cudaGetLastError());
         } else if (few) {
             // one packet's walk, its pairs sorted by leaf into the near pairs' place; these take the list's
@@ -869,7 +875,7 @@ static gwn_status enqueue_chunk(gwn_model_s* m, const void* pts, int dtype, size
             k_few_eval<<<(unsigned)(sms * 8), B, 0, st>>>(m->tree, ws.spos, ws.counters, ws.pairs, ws.wacc, ws.st,
                                                           ws.pairs64, near_cap, p.work);
             if (prof) GWN_CUDA_TRY(cudaEventRecord(ev[3], st));
-            k_pair_eval64_warp<float><<<(unsigned)(sms * 2), B, 0, st>>>(m->tree, ws.spos, near_cap, ws.counters, ws.pairs64,
+            k_pair_eval64_warp<<<(unsigned)(sms * 2), B, 0, st>>>(m->tree, ws.spos, near_cap, ws.counters, ws.pairs64,
                                                                          ws.wacc, ws.st);
             if ((long long)n * m->host.n_leaves > few_cap)
                 k_overflow3<<<1, B, 0, st>>>(m->tree, ws.spos, p.beta2, ws, ws.olist);
@@ -963,7 +969,7 @@ static gwn_status enqueue_chunk(gwn_model_s* m, const void* pts, int dtype, size
             // the near band of both passes in one launch: a point of the second pass has entered it
             // only where the near band's list was full, and then it overflows in the second
             // pass too, so every listed point's FP32 sum is final here or k_overflow3's
-            k_pair_eval64_warp<float><<<(unsigned)(sms * 2), B, 0, st>>>(m->tree, ws.spos, ws.near_cap, ws.counters, ws.pairs64,
+            k_pair_eval64_warp<<<(unsigned)(sms * 2), B, 0, st>>>(m->tree, ws.spos, ws.near_cap, ws.counters, ws.pairs64,
                                                                   ws.wacc, ws.st);
             if (may_overflow || (long long)n * m->host.n_leaves > ws.near_cap)
                 k_overflow3<<<(unsigned)(sms * 2), B, 0, st>>>(m->tree, ws.spos, p.beta2, ws,
@@ -974,7 +980,7 @@ static gwn_status enqueue_chunk(gwn_model_s* m, const void* pts, int dtype, size
         const bool two = m->dim == 2;
         k_finish<float><<<nb, B, 0, st>>>(ni, ws.spos, two ? ws.part : ws.wacc, ws.st, p.precision, p.band, out_w, out_label,
                                           out_status, ws.rlist, rcount, (int)off, ws.rlist_g, ws.gcount, ws.rcap,
-                                          two ? m->cut_size[level] : 0, ws.near);
+                                          two ? m->cut_size[level] : 0, two ? ws.near : nullptr);
         GWN_CUDA_TRY(cudaGetLastError());
         }
     }
@@ -1556,9 +1562,9 @@ __global__ void __launch_bounds__(128) k_query_noalloc2(DevTree t, const void* p
 // 3D: one warp per point with the far exact leaves in place (k_wide3), the near ones
 // through a list, kNoAllocStep points at a time so that everything fits the
 // fixed scratch: per point 16 bytes of position, 4 + 4 + 4 + 4 of sums, status and
-// lists, 4 of FP64 status, 8 near pairs and 3 near-band pairs of 8 bytes (points with more are
-// evaluated by one thread, k_overflow3; the repair's sums follow in the place of the third
-// near-band pair): 124 bytes.  100,000
+// lists, 4 of FP64 status, 8 of near sums, 7 near pairs and 3 near-band pairs of 8 bytes (points
+// with more are evaluated by one thread, k_overflow3; the repair's sums follow in the place of
+// the third near-band pair): 124 bytes.  100,000
 // points on 1.4k leaves, one thread per point with its leaves in place before: 44 ms.
 constexpr size_t kNoAllocStep = 32768;
 static_assert(kNoAllocStep * 124 + 4096 <= sizeof(int) * kNoAllocMaxPoints, "the no-alloc scratch holds one step");
@@ -1577,8 +1583,9 @@ gwn_status noalloc_3d(gwn_model_s* m, const QueryParams& p, const void* points, 
     ws.gcount = scratch + kCounterCount;
     ws.found = (unsigned long long*)(scratch + 2 * kCounterCount);
     ws.spos = (float4*)carve(C * 16);
-    ws.pairs2 = (int2*)carve(C * 64);
-    ws.slow_cap = (long long)C * 8;
+    ws.near = (long long*)carve(C * 8);
+    ws.pairs2 = (int2*)carve(C * 56);
+    ws.slow_cap = (long long)C * 7;
     ws.pairs64 = (int2*)carve(C * 24);
     ws.rw = (double*)(ws.pairs64 + 2 * C);
     ws.wacc = (float*)carve(C * 4);
@@ -1600,19 +1607,19 @@ gwn_status noalloc_3d(gwn_model_s* m, const QueryParams& p, const void* points, 
         // the array keeps the previous call's contents: the counters must start at zero
         GWN_CUDA_TRY(cudaMemsetAsync(scratch, 0, kNoAllocHeader * sizeof(int), st));
         k_scatter_points<3><<<nb, B, 0, st>>>(pts, dtype, c, nullptr, nullptr, ws.spos, ws.wacc, ws.st,
-                                              nullptr);
+                                              ws.near);
         (o3 ? k_wide3<true, false, false> : k_wide3<false, false, false>)
             <<<(unsigned)std::min(((size_t)c + 3) / 4, (size_t)sms * 16), B, 0, st>>>(
                 m->tree, ws.spos, c, nullptr, nullptr, p.beta2, p.beta2_leaf, ws, ws.pairs2, ws.slow_cap, ws.olist2, nullptr,
                 Dense{nullptr, 0}, false);
-        k_pair_eval<float><<<(unsigned)(sms * kEvalBlocks), B, 0, st>>>(m->tree, ws.spos, ws.slow_cap, ws.counters + 8, ws.counters,
-                                                              ws.pairs2, ws.wacc, ws.st, ws.pairs64, near_cap,
-                                                              ws.olist2, nullptr);
-        k_pair_eval64_warp<float><<<(unsigned)(sms * 2), B, 0, st>>>(m->tree, ws.spos, near_cap, ws.counters, ws.pairs64,
-                                                                     ws.wacc, ws.st);
-        k_overflow3<<<(unsigned)(sms * 2), B, 0, st>>>(m->tree, ws.spos, p.beta2, ws, ws.olist2);
+        k_pair_eval<long long><<<(unsigned)(sms * kEvalBlocks), B, 0, st>>>(
+            m->tree, ws.spos, ws.slow_cap, ws.counters + 8, ws.counters, ws.pairs2, ws.near, ws.st, ws.pairs64, near_cap,
+            ws.olist2, nullptr);
+        k_pair_eval64_warp<<<(unsigned)(sms * 2), B, 0, st>>>(m->tree, ws.spos, near_cap, ws.counters, ws.pairs64, ws.wacc,
+                                                              ws.st, ws.near);
+        k_overflow3<<<(unsigned)(sms * 2), B, 0, st>>>(m->tree, ws.spos, p.beta2, ws, ws.olist2, ws.near);
         k_finish<float><<<nb, B, 0, st>>>(c, ws.spos, ws.wacc, ws.st, p.precision, p.band, w, label, status, nullptr, nullptr,
-                                          0, ws.rlist_g, ws.gcount, c);
+                                          0, ws.rlist_g, ws.gcount, c, 0, ws.near);
         const RepairList R{ws.rlist_g, ws.gcount, c, ws.rw, ws.rst};
         k_rtrav_warp<true><<<(unsigned)(sms * 4), 32 * kRepairWarps, 0, st>>>(
             m->tree, pts, dtype, p.beta2_repair, R, p.beta2_repair, Rule64{kRatio64Repair, false}, false);

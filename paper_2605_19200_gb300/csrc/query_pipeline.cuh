@@ -31,6 +31,15 @@
 
 namespace gwn {
 
+// Sums that do not depend on the order of their additions (direct sum, no-alloc query): in units of
+// 2^-44 (rounding 2.8e-14, where an FP32 leaf's is 1e-9 and more; a total of up to 5e5),
+// what is not finite in `rest`
+constexpr float kSumUnit = 17592186044416.f;  // 2^44
+__device__ __forceinline__ void add_fixed(long long* sum, float* rest, int i, double v) {
+    if (isfinite(v)) atomicAdd(reinterpret_cast<unsigned long long*>(&sum[i]), (unsigned long long)__double2ll_rn(v * (double)kSumUnit));
+    else atomicAdd(&rest[i], (float)v);
+}
+
 constexpr int kBinBits2 = 9;   // 512 x 512 cells in 2D
 constexpr int kBinBits3 = 5;   // 32^3 cells in 3D (default; the autotuner picks 4, 5 or 6 per model)
 constexpr int kMaxBinCells = 1 << 18;  // 2^(2 x 9) = 2^(3 x 6)
@@ -213,8 +222,8 @@ __global__ void k_scatter_points(const void* pts, int dtype, int n, const int* k
     load_point_f(pts, dtype, DIM, i, q);
     const int pos = key ? atomicAdd(&cursor[key[i]], 1) : i;  // no key: the caller's order (few points)
     spos[pos] = make_float4(q[0], q[1], q[2], __int_as_float(i));
-    if (DIM == 2) near[i] = 0;
-    else wacc[i] = 0.f;  // the warps of a split packet add to these
+    if (near) near[i] = 0;
+    if (DIM == 3) wacc[i] = 0.f;  // the warps of a split packet add to these
     st[i] = 0u;
 }
 
@@ -856,13 +865,14 @@ __global__ void __launch_bounds__(128) k_wide3(DevTree t, const float4* spos, in
 // points whose pairs still overflowed after the last round: whole traversal
 // again, leaves in place
 __global__ void __launch_bounds__(128) k_overflow3(DevTree t, const float4* spos, float beta2, Workspace ws,
-                                                   const int* list) {
+                                                   const int* list, long long* near = nullptr) {
     int cnt = ws.counters[3];
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < cnt; k += gridDim.x * blockDim.x) {
         int qi = list[k];
         const float4 p = spos[qi];
         uint32_t st = 0;
         ws.wacc[qi] = query3_32(t, p.x, p.y, p.z, beta2, st);
+        if (near) near[qi] = 0;
         ws.st[qi] = st;
     }
 }
@@ -1029,9 +1039,10 @@ __global__ void __launch_bounds__(128) k_pair_fast2(DevTree t, const float4* spo
 // The direct sum's far pairs (every leaf for every point, summed in FP64 so that the
 // thousands of additions do not round): a block holds 128 points and walks one of
 // gridDim.y slices of the leaves, whose tables it reads at the same address in
-// all lanes.  Near and deeper pairs go to `slow` (k_pair_eval), points whose slow
-// pairs do not fit to olist (k_direct_overflow3).  acc and st zeroed beforehand.
-__global__ void __launch_bounds__(128) k_direct3(DevTree t, const float4* spos, int n, double* acc, uint32_t* st,
+// all lanes; the slices' sums add up in fixed point (add_fixed).  Near and deeper pairs go to
+// `slow` (k_pair_eval), points whose slow pairs do not fit to olist (k_direct_overflow3).  acc,
+// rest and st zeroed beforehand.
+__global__ void __launch_bounds__(128) k_direct3(DevTree t, const float4* spos, int n, long long* acc, float* rest, uint32_t* st,
                                                  int* counters, int2* slow, long long slow_cap, int* olist) {
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
@@ -1060,11 +1071,11 @@ __global__ void __launch_bounds__(128) k_direct3(DevTree t, const float4* spos, 
             }
         }
     }
-    if (act) atomicAdd(&acc[i], sum);
+    if (act) add_fixed(acc, rest, i, sum);
 }
 
 // direct sums whose near pairs did not fit the list: one thread per point
-__global__ void __launch_bounds__(128) k_direct_overflow3(DevTree t, const float4* spos, double* acc, uint32_t* stv,
+__global__ void __launch_bounds__(128) k_direct_overflow3(DevTree t, const float4* spos, long long* acc, float* rest, uint32_t* stv,
                                                           const int* counters, const int* olist) {
     const int cnt = counters[3];
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < cnt; k += gridDim.x * blockDim.x) {
@@ -1073,7 +1084,9 @@ __global__ void __launch_bounds__(128) k_direct_overflow3(DevTree t, const float
         double w = 0.0;
         uint32_t st = 0;
         for (int l = 0; l < t.n_leaves; ++l) w += (double)leaf3_eval32(t, l, p.x, p.y, p.z, st);
-        acc[i] = w;
+        acc[i] = 0;
+        rest[i] = 0.f;
+        add_fixed(acc, rest, i, w);
         stv[i] = st;
     }
 }
@@ -1086,29 +1099,34 @@ __global__ void __launch_bounds__(128) k_direct_overflow3(DevTree t, const float
 //      foot-point search;
 //   2. one thread per listed search (leaf_hit_solve), and one thread per pair for
 //      the level-0 panels of its curves from the FP32 node tables; the halves of the
-//      curves that need shorter panels are listed;
+//      curves that need shorter panels are listed (a thread that finds the list full
+//      goes on from that curve once the listed halves are done);
 //   3. one thread per listed half: its level-1 panel from the table; those that need
-//      shorter ones list their two panels of level 2;
-//   4. rounds over the listed panels, four lanes to a panel (one Gauss-Legendre node
-//      each, from the curve's Bernstein form): the integral, or two panels of
-//      the next level for the next round.
+//      shorter ones push their two panels of level 2;
+//   4. steps of up to kNearTake panels from the top of that stack, four lanes to a panel (one
+//      Gauss-Legendre node each, from the curve's Bernstein form): the integral, or two
+//      panels of the next level onto the stack.
 // Pairs FP32 cannot resolve go to the FP64 near band; where its list is full their point goes
 // to olist (the points evaluated again in place), or, without one, is flagged for the repair.
-// One thread doing all of this for its pair from the Bernstein form alone (28 D + 70 flops per node, the tables 34) took
-// 5.8 ms on 1.3M points of a 4.7k-leaf model, whole curves below level 1 per
+// One thread doing all of this for its pair from the Bernstein form alone (28 D + 70 flops per node, the
+// tables 34) took 5.8 ms on 1.3M points of a 4.7k-leaf model, whole curves below level 1 per
 // thread 1.8 ms with 10 to 12 active lanes per instruction.
-constexpr int kNearHalves = 2048, kNearPanels = 1024;
-template <typename Acc>  // float, or double (the direct sum)
+// Acc: float (the traversal, onto wacc), or long long, whose sums -- a pair's panels and a
+// point's pairs -- add up in fixed point, so that two runs give the same bits whatever
+// the order of the list (the direct sum and the no-alloc query).
+constexpr int kNearHalves = 2048, kNearPanels = 2048, kNearStep = 512, kNearTake = 256;
+template <typename Acc>
 __global__ void __launch_bounds__(128, 5) k_pair_eval(DevTree t, const float4* spos, long long npair_cap,
                                                    const int* count, int* counters, const int2* pairs, Acc* wacc,
                                                    uint32_t* st, int2* pairs64, int npair64_cap, int* olist,
                                                    unsigned long long* work) {
-    __shared__ float sq[3][128], ss[3][128], sacc[128];
+    constexpr bool kFixed = sizeof(Acc) == 8;
+    __shared__ Acc sacc[128];
+    __shared__ float sq[3][128], ss[3][128];
     __shared__ int sleaf[128], sfail[128], shit[128];
-    // the halves (phase 3), then the panels of alternating rounds (phase 4):
     // pair | panel index | level | curve, 7 + 10 + 4 + 10 bits
-    __shared__ unsigned stask[kNearHalves], spanel[kNearPanels];
-    __shared__ int nhit, nhalf, npanel[2];
+    __shared__ unsigned stask[kNearHalves], spanel[kNearPanels], schild[2 * kNearTake];
+    __shared__ int nhit, nhalf, npanel, nchild;
     constexpr int kMaxCurve = 1 << 10;
     WorkLocal wl = {};
     const int tid = threadIdx.x, lane = tid & 31;
@@ -1117,6 +1135,14 @@ __global__ void __launch_bounds__(128, 5) k_pair_eval(DevTree t, const float4* s
     const long long np = min((long long)*count, npair_cap);
     auto entry = [](int o, int c, int level, unsigned idx) {
         return (unsigned)o | idx << 7 | (unsigned)level << 17 | (unsigned)c << 21;
+    };
+    auto add = [&](int o, float v) {
+        if constexpr (kFixed) {
+            if (isfinite(v)) atomicAdd(reinterpret_cast<unsigned long long*>(&sacc[o]), (unsigned long long)__float2ll_rn(v * kSumUnit));
+            else sfail[o] = 1;
+        } else {
+            atomicAdd(&sacc[o], v);
+        }
     };
     // panel idx of `level` of curve c of the leaf of pair o and what is below it, by one thread
     auto whole_panel = [&](int o, int c, int level, unsigned idx) {
@@ -1129,12 +1155,12 @@ __global__ void __launch_bounds__(128, 5) k_pair_eval(DevTree t, const float4* s
         bool deep = false;
         for (unsigned j = idx << sub; j < ((idx + 1) << sub); ++j)
             a += panel_subtree<float>(g, ci.deg, q, s, l0, j, kLevel32, kRatio32, deep, work ? &wl : nullptr);
-        atomicAdd(&sacc[o], ci.mult * a * inv4pi);
+        add(o, ci.mult * a * inv4pi);
         if (deep) sfail[o] = 1;
     };
     for (long long base = (long long)blockIdx.x * 128; base < np; base += (long long)gridDim.x * 128) {
-        if (tid == 0) nhit = nhalf = npanel[0] = npanel[1] = 0;
-        sacc[tid] = 0.f;
+        if (tid == 0) nhit = nhalf = npanel = nchild = 0;
+        sacc[tid] = 0;
         sfail[tid] = 0;
         __syncthreads();
         bool act = base + tid < np;
@@ -1182,12 +1208,14 @@ __global__ void __launch_bounds__(128, 5) k_pair_eval(DevTree t, const float4* s
             float hits = 0.f;
             const int hr = leaf_hit_solve<float>(t, I, g, qo, I.nrm, e1, e2, sig, hit_tau_eps<float>(I.diag), &hits, kNear32);
             if (hr == kHitUnsure) sfail[o] = 1;
-            else if (hr == kHitOk) atomicAdd(&sacc[o], -hits);
+            else if (hr == kHitOk) add(o, -hits);
         }
-        if (act) {
-            const int2 range = __ldg(t.lrange + pr.y);
+        const int2 range = act ? __ldg(t.lrange + pr.y) : make_int2(0, 0);
+        int c = 0;  // next curve
+        bool more;
+        do {
             float acc = 0.f;
-            for (int c = 0; c < range.y; ++c) {
+            for (; c < range.y; ++c) {
                 const float4* H = t.c3n + (size_t)(range.x + c) * kC3NodeVec;
                 const float4 hd = __ldg(H);
                 if (hd.x < kInfF) {
@@ -1195,106 +1223,116 @@ __global__ void __launch_bounds__(128, 5) k_pair_eval(DevTree t, const float4* s
                     fast_panel(H + 1, q, s, pa, da);
                     if (work) wl.v[kWorkFastNodes] += 4;
                     if (hd.x * hd.x <= ratio2 * da) {
-                        acc += hd.w * pa;
+                        if constexpr (kFixed) add(tid, hd.w * pa * inv4pi);
+                        else acc += hd.w * pa;
                         continue;
                     }
                 }
-                const int slot = c < kMaxCurve ? atomicAdd(&nhalf, 2) : kNearHalves;
-                for (int j = 0; j < 2; ++j) {
-                    if (slot + j < kNearHalves) stask[slot + j] = entry(tid, c, 1, j);
-                    else whole_panel(tid, c, 1, j);  // list full
-                }
-            }
-            atomicAdd(&sacc[tid], acc * inv4pi);
-        }
-        __syncthreads();
-        // level 1, one thread per half curve
-        const int nh = min(nhalf, kNearHalves);
-        for (int j = tid; j < nh; j += 128) {
-            const unsigned e = stask[j];
-            const int o = e & 127, half = e >> 7 & 1, c = e >> 21;
-            const int k = t.lrange[sleaf[o]].x + c;
-            const float4* H = t.c3n + (size_t)k * kC3NodeVec;
-            const float4 hd = __ldg(H);
-            const float len = half ? hd.z : hd.y;
-            if (len < kInfF) {
-                const float qo[3] = {sq[0][o], sq[1][o], sq[2][o]}, so[3] = {ss[0][o], ss[1][o], ss[2][o]};
-                float pa, da;
-                fast_panel(H + 7 + 6 * half, qo, so, pa, da);
-                if (work) wl.v[kWorkFastNodes] += 4;
-                if (len * len <= ratio2 * da) {
-                    atomicAdd(&sacc[o], 0.5f * hd.w * pa * inv4pi);
+                if (c >= kMaxCurve) {
+                    for (int j = 0; j < 2; ++j) whole_panel(tid, c, 1, j);
                     continue;
                 }
+                const int slot = atomicAdd(&nhalf, 2);
+                if (slot >= kNearHalves) break;  // full: this curve in the next turn
+                for (int j = 0; j < 2; ++j) stask[slot + j] = entry(tid, c, 1, j);
             }
-            // level 2 (or the curve's own first level): listed, or by this thread
-            const int slot = t.c3[k].min_level <= 2 ? atomicAdd(&npanel[0], 2) : kNearPanels;
-            for (int i = 0; i < 2; ++i) {
-                if (slot + i < kNearPanels) spanel[slot + i] = entry(o, c, 2, 2 * half + i);
-                else whole_panel(o, c, 2, 2 * half + i);
+            if constexpr (!kFixed) {
+                if (act) atomicAdd(&sacc[tid], acc * inv4pi);
             }
-        }
-        __syncthreads();
-        // rounds: panels of round r in spanel (even) or the first kNearPanels of stask (odd)
-        for (int r = 0;; ++r) {
-            const int n = min(npanel[r & 1], kNearPanels);
-            if (n == 0) break;
-            const unsigned* in = r & 1 ? stask : spanel;
-            unsigned* out = r & 1 ? spanel : stask;
-            for (int j0 = 0; j0 < n; j0 += 32) {
-                const int j = j0 + (tid >> 2), node = tid & 3;
-                const bool on = j < n;
-                float f = 0.f, dm = 1e30f, x[3] = {0, 0, 0};
-                unsigned e = 0;
-                Curve3Info ci{0, 1, 0.f, 0};
-                float h = 1.f;
-                if (on) {
-                    e = in[j];
-                    const int o = e & 127;
-                    ci = t.c3[t.lrange[sleaf[o]].x + (int)(e >> 21)];
-                    const Geo32 g{nullptr, t.c3pts + ci.ctrl_off};
-                    const float qo[3] = {sq[0][o], sq[1][o], sq[2][o]}, so[3] = {ss[0][o], ss[1][o], ss[2][o]};
-                    h = 1.f / (float)(1u << (e >> 17 & 15));
-                    f = Gl8<float>::w(node) *
-                        gl_node_any<float>(g, ci.deg, (float)(e >> 7 & 1023) * h + h * Gl8<float>::x(node), qo, so, x, &dm);
-                    if (work) {
-                        wl.v[kWorkGlNodes] += 1;
-                        wl.v[kWorkGlDeg] += ci.deg;
-                    }
-                }
-                const unsigned full = 0xffffffffu;
-                const float e0 = x[0] - __shfl_up_sync(full, x[0], 1), e1 = x[1] - __shfl_up_sync(full, x[1], 1),
-                            e2 = x[2] - __shfl_up_sync(full, x[2], 1);
-                float len = node ? Num<float>::sqrt_fast(e0 * e0 + e1 * e1 + e2 * e2) : 0.f;
-                for (int off = 1; off < 4; off <<= 1) {
-                    f += __shfl_xor_sync(full, f, off);
-                    len += __shfl_xor_sync(full, len, off);
-                    dm = fminf(dm, __shfl_xor_sync(full, dm, off));
-                }
-                len *= Gl8<float>::span_inv;
-                if (on && node == 0) {
-                    const int o = e & 127, level = e >> 17 & 15;
-                    const unsigned idx = e >> 7 & 1023;
-                    const bool refine = len * len > ratio2 * dm;
-                    if (!refine || level >= kLevel32) {
-                        atomicAdd(&sacc[o], ci.mult * f * h * inv4pi);
-                        if (refine) sfail[o] = 1;
-                    } else {
-                        const int slot = atomicAdd(&npanel[(r + 1) & 1], 2);
-                        for (int i = 0; i < 2; ++i) {
-                            if (slot + i < kNearPanels) out[slot + i] = entry(o, e >> 21, level + 1, 2 * idx + i);
-                            else whole_panel(o, e >> 21, level + 1, 2 * idx + i);
+            __syncthreads();
+            const int nh = min(nhalf, kNearHalves);
+            for (int h0 = 0; h0 < nh; h0 += kNearStep) {
+                // level 1, one thread per half curve; the stack is empty
+                for (int j = h0 + tid; j < min(nh, h0 + kNearStep); j += 128) {
+                    const unsigned e = stask[j];
+                    const int o = e & 127, half = e >> 7 & 1, cj = e >> 21;
+                    const int k = t.lrange[sleaf[o]].x + cj;
+                    const float4* H = t.c3n + (size_t)k * kC3NodeVec;
+                    const float4 hd = __ldg(H);
+                    const float len = half ? hd.z : hd.y;
+                    if (len < kInfF) {
+                        const float qo[3] = {sq[0][o], sq[1][o], sq[2][o]}, so[3] = {ss[0][o], ss[1][o], ss[2][o]};
+                        float pa, da;
+                        fast_panel(H + 7 + 6 * half, qo, so, pa, da);
+                        if (work) wl.v[kWorkFastNodes] += 4;
+                        if (len * len <= ratio2 * da) {
+                            add(o, 0.5f * hd.w * pa * inv4pi);
+                            continue;
                         }
                     }
+                    // level 2; by this thread where the curve's own first level is lower
+                    if (t.c3[k].min_level <= 2) {
+                        const int slot = atomicAdd(&npanel, 2);
+                        for (int i = 0; i < 2; ++i) spanel[slot + i] = entry(o, cj, 2, 2 * half + i);
+                    } else {
+                        for (int i = 0; i < 2; ++i) whole_panel(o, cj, 2, 2 * half + i);
+                    }
+                }
+                __syncthreads();
+                int sp = npanel;  // block-uniform
+                while (sp > 0) {
+                    const int take = stack_take(sp, kNearTake, kNearPanels);
+                    for (int j0 = 0; j0 < take; j0 += 32) {
+                        const int j = j0 + (tid >> 2), node = tid & 3;
+                        const bool on = j < take;
+                        float f = 0.f, dm = 1e30f, x[3] = {0, 0, 0};
+                        unsigned e = 0;
+                        Curve3Info ci{0, 1, 0.f, 0};
+                        float h = 1.f;
+                        if (on) {
+                            e = spanel[sp - take + j];
+                            const int o = e & 127;
+                            ci = t.c3[t.lrange[sleaf[o]].x + (int)(e >> 21)];
+                            const Geo32 g{nullptr, t.c3pts + ci.ctrl_off};
+                            const float qo[3] = {sq[0][o], sq[1][o], sq[2][o]}, so[3] = {ss[0][o], ss[1][o], ss[2][o]};
+                            h = 1.f / (float)(1u << (e >> 17 & 15));
+                            f = Gl8<float>::w(node) * gl_node_any<float>(g, ci.deg, (float)(e >> 7 & 1023) * h + h * Gl8<float>::x(node),
+                                                                         qo, so, x, &dm);
+                            if (work) {
+                                wl.v[kWorkGlNodes] += 1;
+                                wl.v[kWorkGlDeg] += ci.deg;
+                            }
+                        }
+                        const unsigned full = 0xffffffffu;
+                        const float e0 = x[0] - __shfl_up_sync(full, x[0], 1), e1 = x[1] - __shfl_up_sync(full, x[1], 1),
+                                    e2 = x[2] - __shfl_up_sync(full, x[2], 1);
+                        float len = node ? Num<float>::sqrt_fast(e0 * e0 + e1 * e1 + e2 * e2) : 0.f;
+                        for (int off = 1; off < 4; off <<= 1) {
+                            f += __shfl_xor_sync(full, f, off);
+                            len += __shfl_xor_sync(full, len, off);
+                            dm = fminf(dm, __shfl_xor_sync(full, dm, off));
+                        }
+                        len *= Gl8<float>::span_inv;
+                        if (on && node == 0) {
+                            const int o = e & 127, level = e >> 17 & 15;
+                            const unsigned idx = e >> 7 & 1023;
+                            const bool refine = len * len > ratio2 * dm;
+                            if (!refine || level >= kLevel32) {
+                                add(o, ci.mult * f * h * inv4pi);
+                                if (refine) sfail[o] = 1;
+                            } else {
+                                const int slot = atomicAdd(&nchild, 2);
+                                for (int i = 0; i < 2; ++i) schild[slot + i] = entry(o, e >> 21, level + 1, 2 * idx + i);
+                            }
+                        }
+                    }
+                    __syncthreads();
+                    const int k = nchild;
+                    sp -= take;
+                    for (int j = tid; j < k; j += 128) spanel[sp + j] = schild[j];
+                    sp += k;
+                    __syncthreads();
+                    if (tid == 0) nchild = npanel = 0;
+                    __syncthreads();
                 }
             }
-            __syncthreads();
-            if (tid == 0) npanel[r & 1] = 0;
-            __syncthreads();
-        }
+            if (tid == 0) nhalf = 0;
+            more = __syncthreads_or(c < range.y);
+        } while (more);
         if (act) {
             if (!sfail[tid]) {
-                atomicAdd(&wacc[pr.x], (Acc)sacc[tid]);
+                if constexpr (kFixed) atomicAdd(reinterpret_cast<unsigned long long*>(&wacc[pr.x]), (unsigned long long)sacc[tid]);
+                else atomicAdd(&wacc[pr.x], sacc[tid]);
             } else {
                 const int slot = atomicAdd(&counters[2], 1);
                 if (slot < npair64_cap) {
@@ -1324,11 +1362,11 @@ __device__ __forceinline__ bool leaf_fits_w4(const DevTree& t, int li) {
     return dmax <= 6;
 }
 
-// the near band with one warp per pair (leaf3_warp64)
-template <typename Acc>
+// the near band with one warp per pair (leaf3_warp64), onto near in fixed point where given, else
+// onto wacc
 __global__ void __launch_bounds__(128) k_pair_eval64_warp(DevTree t, const float4* spos, int npair64_cap,
-                                                          const int* counters, const int2* pairs64, Acc* wacc,
-                                                          uint32_t* st) {
+                                                          const int* counters, const int2* pairs64, float* wacc,
+                                                          uint32_t* st, long long* near = nullptr) {
     __shared__ int2 sstk[4][kQuadStack];
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int np = min(counters[2], npair64_cap);
@@ -1342,7 +1380,8 @@ __global__ void __launch_bounds__(128) k_pair_eval64_warp(DevTree t, const float
         const bool ok = leaf_fits_w4(t, pr.y) ? leaf3_warp64<4>(t, pr.y, q, kRatio64BandW4, kLevel64, sstk[wid], &v)
                                               : leaf3_warp64<8>(t, pr.y, q, kRatio64Band, kLevel64, sstk[wid], &v);
         if (lane == 0) {
-            atomicAdd(&wacc[pr.x], ok ? (Acc)(float)v : (Acc)0);
+            if (ok && near) add_fixed(near, wacc, pr.x, (double)(float)v);
+            else if (ok) atomicAdd(&wacc[pr.x], (float)v);
             if (!ok) atomicOr(&st[pr.x], GWN_QS_UNRESOLVED);
         }
         __syncwarp();
@@ -1352,7 +1391,7 @@ __global__ void __launch_bounds__(128) k_pair_eval64_warp(DevTree t, const float
 // outputs of one chunk (points off .. off + n - 1 of the query); points to
 // repair go to the query's list (index off + i) while it has room, else to the
 // chunk's own list (index i), repaired right after the chunk
-// parts > 0 (2D): wacc holds the subtrees' sums (value2)
+// parts > 0 (2D): wacc holds the subtrees' sums (value2); near: sums in fixed point
 template <typename Acc>
 __global__ void k_finish(int n, const float4* spos, const Acc* wacc, const uint32_t* stv, int precision, float band, double* out_w,
                          int* out_label, uint32_t* out_status, int* rlist, int* rcount, int off, int* rlist_g,
@@ -1361,6 +1400,7 @@ __global__ void k_finish(int n, const float4* spos, const Acc* wacc, const uint3
     if (k >= n) return;
     const int i = __float_as_int(spos[k].w);  // place in the binned copy -> the caller's order
     double w = sizeof(Acc) == 4 && parts ? (double)value2(reinterpret_cast<const float*>(wacc), near, n, parts, k)
+               : near                    ? (double)wacc[k] + (double)near[k] * (1.0 / (double)kSumUnit)
                                          : (double)wacc[k];
     uint32_t st = stv[k];
     if (precision == GWN_PREC_FP32_REPAIR) {

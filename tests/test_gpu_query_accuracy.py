@@ -201,3 +201,25 @@ def test_small_queries_keep_a_small_workspace():
     gwn.gwn_query(m, q, out=out)
     torch.cuda.synchronize()
     assert before - torch.cuda.mem_get_info()[0] <= 128 << 20
+
+
+@pytest.mark.parametrize("call", ["direct", "noalloc"])
+@pytest.mark.parametrize("kind", ["cad", "round"])
+def test_two_runs_give_the_same_bits(call, kind):
+    """The FP32 direct sum and the no-alloc call at points next to the faces, where each point has several
+    near pairs whose order in the lists differs from run to run."""
+    patches = configs.cad_3d(seed=5, n_patches=60)[0] if kind == "cad" else configs.sphere_3d(cells=2, n_queries=1)[0]
+    n = 20001
+    pts = torch.from_numpy(np.concatenate([_on_faces(patches, n // 2, 11, 1e-5), _on_faces(patches, n - n // 2, 12, 1e-3)])).cuda()
+    m = gwn.gwn_build_3d(patches, beta=6.0, beta_leaf=4.0)
+
+    def run():
+        if call == "direct":
+            return m.query(pts, mode=gwn.MODE_DIRECT, precision=gwn.PREC_FP32)
+        return gwn.api.gwn_query_noalloc(m, pts, (torch.empty(n, dtype=torch.float64, device="cuda"), None,
+                                                  torch.empty(n, dtype=torch.int32, device="cuda")))
+    w, _, st = run()
+    assert int((st & gwn.QS_NEAR).ne(0).sum()) > n // 8
+    for _ in range(5):
+        w2, _, st2 = run()
+        assert torch.equal(w, w2) and torch.equal(st, st2)
