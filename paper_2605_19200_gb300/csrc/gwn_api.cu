@@ -1194,9 +1194,10 @@ static gwn_status autotune(gwn_model_s* m) {
                 s = fail(GWN_ERR_CUDA, "autotune readback failed");
                 break;
             }
-            // a candidate whose exact-leaf pairs overflow the work list is rejected:
-            // its overflow path is slow and not counted
-            if (acc[3] + acc[6] > 0) continue;
+            // a candidate whose exact-leaf pairs overflow the work list is rejected (its
+            // overflow path is slow and not counted), and so is one with so many that its
+            // leaves took beta
+            if (acc[3] + acc[6] > 0 || (d == 3 && acc[0] > dense_limit(m->ws, nv))) continue;
             if (e < fb_err) {
                 fb_err = e;
                 fb_b = b;
