@@ -914,12 +914,17 @@ static gwn_status enqueue_chunk(gwn_model_s* m, const void* pts, int dtype, size
                 k<<<blocks, B, 0, st>>>(m->tree, ws.spos, ni, idx, n_dev, p.beta2, p.beta2_leaf, ws, ws.pairs2,
                                         ws.slow_cap, list ? ws.olist : ws.olist2, p.work, d, again);
             };
+            // (the second walk of a dense chunk split to about one wave of warps: its blocks are
+            // launched for every chunk that could be dense)
+            int level_again = 0;
+            while (level_again < level && ((size_t)packets << (level_again + 1)) <= (size_t)28 * sms) ++level_again;
             auto packet_pass = [&](Dense d, bool again) {
+                const int lv = again ? level_again : level;
                 auto trav = p.work ? (o3 ? k_trav3<true, true> : k_trav3<false, true>)
                                    : (o3 ? k_trav3<true, false> : k_trav3<false, false>);
-                trav<<<dim3(packets, (unsigned)m->cut_size[level]), 32, trav3_smem(m->stack_depth), st>>>(
-                    m->tree, ws.spos, ni, p.beta2, again ? p.beta2 : p.beta2_leaf, m->stack_depth, m->cuts[level], ws,
-                    p.work, ws.olist, d, again);
+                trav<<<dim3(packets, (unsigned)m->cut_size[lv]), 32, trav3_smem(m->stack_depth), st>>>(
+                    m->tree, ws.spos, ni, p.beta2, again ? p.beta2 : p.beta2_leaf, m->stack_depth, m->cuts[lv], ws, p.work,
+                    ws.olist, d, again);
             };
             auto eval_pass = [&](int* olist) {
                 k_pair_eval<float><<<(unsigned)(sms * kEvalBlocks), B, 0, st>>>(m->tree, ws.spos, ws.slow_cap, ws.counters + 8,
