@@ -551,6 +551,7 @@ size_t workspace_layout(int dim, int n_leaves, size_t n, char* base, Workspace* 
     w.rlist_g = (int*)carve(n * sizeof(int));
     w.rst = (uint32_t*)carve(n * sizeof(uint32_t));
     w.rcap = (int)n;
+    w.list_points = (int)n;
     w.olist = (int*)carve(n * sizeof(int));
     w.olist2 = (int*)carve((dim != 2 ? n : 0) * sizeof(int));
     w.work = (unsigned long long*)carve(kWorkCount * sizeof(unsigned long long));
@@ -643,7 +644,7 @@ static int bin_bits3(size_t n, int ppc) {
 // error 1.4e-5 at beta_leaf, 2.2e-6 at beta.
 static unsigned long long dense_limit(const Workspace& ws, size_t n) {
     const double lists = std::min(3.3, std::max(1.4, 1.4 + ((double)n - 150000.0) / 300000.0));
-    return (unsigned long long)(lists * (96.0 * (double)ws.rcap + 65536.0));
+    return (unsigned long long)(lists * (96.0 * (double)ws.list_points + 65536.0));
 }
 
 // the kernels' parameters of one query
@@ -1471,6 +1472,7 @@ gwn_status gwn_query(gwn_model m, const void* points, int32_t dtype, int32_t mem
     size_t obytes = n * (sizeof(double) + sizeof(int32_t) + sizeof(uint32_t));
     gwn_status s = ensure_workspace(m, n, mem == GWN_MEM_HOST ? pbytes + obytes + 64 : 0);
     if (s != GWN_OK) return s;
+    m->ws.list_points = (int)std::min(std::max<size_t>(n, 4096), kChunk);
     // calls on other streams share the model's workspace: start after the previous call's work
     if (!m->last) GWN_CUDA_TRY(cudaEventCreateWithFlags(&m->last, cudaEventDisableTiming));
     if (m->last_recorded) GWN_CUDA_TRY(cudaStreamWaitEvent(st, m->last, 0));

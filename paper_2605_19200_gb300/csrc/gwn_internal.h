@@ -292,6 +292,7 @@ struct Workspace {
                       // takes (cleared once per query)
     unsigned* bbox;   // 8: the chunk's bounding box as order-preserving keys (k_bbox)
     int rcap;         // entries of rlist_g (= the points a workspace holds)
+    int list_points;  // points that dense_limit counts for: a query's own where the workspace grew for other queries
     long long pair_cap, slow_cap;
 };
 

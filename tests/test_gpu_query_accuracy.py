@@ -223,3 +223,64 @@ def test_two_runs_give_the_same_bits(call, kind):
     for _ in range(5):
         w2, _, st2 = run()
         assert torch.equal(w, w2) and torch.equal(st, st2)
+
+
+@pytest.mark.parametrize("n", [1, 16, 17, 200, 4097])
+@pytest.mark.parametrize("local_ratio", [0.0, 64.0])
+def test_small_queries_of_round_parts(oracle_lib, n, local_ratio):
+    """Curves of high degree (circular trims) on the small-query paths, with and without packet local
+    expansions (at 64 packet radii their remainder, 64^-3 of a term, is far below the bound)."""
+    from synth import geometry as G
+    patches = configs.sphere_3d(cells=2, n_queries=1)[0]
+    lo, hi = G.shape_bbox_3d(patches)
+    q = np.concatenate([_on_faces(patches, (n + 1) // 2, n, 1e-2),
+                        np.random.default_rng(n).uniform(lo, hi, (n // 2, 3)).astype(np.float32)])
+    m = gwn.gwn_build_3d(patches, beta=6.0, beta_leaf=4.0)
+    w, lab, _ = m.query(torch.from_numpy(q).cuda(), local_ratio=local_ratio)
+    idx = np.unique(np.r_[0, n - 1, np.random.default_rng(1).integers(0, n, 200)])
+    w_ref, _ = oracle_lib.gwn3d(patches, q[idx].astype(np.float64))
+    ok = np.isfinite(w_ref)
+    assert np.max(np.abs(w.cpu().numpy()[idx][ok] - w_ref[ok])) <= 1e-4
+    assert torch.equal(lab, torch.round(w).int())
+
+
+def test_values_do_not_depend_on_earlier_queries():
+    """A crowded query before and after a larger one on the same model: the same terms, up to FP32 sums (5e-6,
+    as above); with its leaves at another factor it would differ by 2e-5."""
+    patches = configs.cad_3d(seed=9, n_patches=330)[0]
+    m = gwn.gwn_build_3d(patches, beta=9.0, beta_leaf=5.5, precision=gwn.PREC_FP32)
+    pts = torch.from_numpy(_on_faces(patches, 9000, 5, 1e-3)).cuda()
+    before = m.query(pts)[0].clone()
+    m.query(torch.from_numpy(_on_faces(patches, 120000, 6, 1e-3)).cuda())
+    assert float((m.query(pts)[0] - before).abs().max()) <= 5e-6
+
+
+def test_concurrent_callers():
+    """Two threads with a stream each, on a model they share and on one of their own, over the paths that
+    keep state in the workspace: values as alone, to the rounding of FP32 sums (as above: 5e-6)."""
+    import threading
+    models = [gwn.gwn_build_3d(configs.cad_3d(seed=9, n_patches=k)[0], beta=9.0, beta_leaf=5.5) for k in (330, 60, 100)]
+    patches = configs.cad_3d(seed=9, n_patches=330)[0]
+    pts = [torch.from_numpy(_on_faces(patches, n, n, 1e-3)).cuda() for n in (9, 900, 9000, 40000)]
+    ref = {(j, k): models[j].query(p)[0] for j in range(3) for k, p in enumerate(pts)}
+    torch.cuda.synchronize()
+    bad = []
+
+    def work(own):
+        stream = torch.cuda.Stream()
+        with torch.cuda.stream(stream):
+            for r in range(6):
+                for k, p in enumerate(pts):
+                    for j in (0, own):
+                        w, _, _ = models[j].query(p)
+                        stream.synchronize()
+                        d = float((w - ref[j, k]).abs().max())
+                        if not d <= 5e-6:
+                            bad.append((j, k, d))
+
+    threads = [threading.Thread(target=work, args=(own,)) for own in (1, 2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not bad
