@@ -155,7 +155,9 @@ typedef struct {
     double beta;        /* 0 = the model's */
     int32_t count_work; /* 1: count algorithmic work units (slower; see gwn_last_query_stats) */
     int32_t profile;    /* 1: time the traversal and exact-leaf kernels with CUDA events on the stream */
-    double beta_leaf;   /* 0 = the model's */
+    double beta_leaf;   /* 0 = the model's; leaves take beta where a 3D query has so many exact
+                           (point, leaf) pairs (from 134 a point on) that their far terms would be most of
+                           the error */
     double repair_band; /* > 0: re-evaluate in FP64 when |w - round(w) +- 1/2| < this band instead of the
                            model's (GWN_PREC_FP32_REPAIR only); 0 = the model's (default 0) */
     double local_ratio; /* 3D, order-2 evaluation: a cluster that every query of a warp's packet (32 binned
@@ -198,7 +200,13 @@ gwn_status gwn_build_3d(const gwn_patch3d* patches, size_t n, const gwn_build_op
  *   stream    : a cudaStream_t, or NULL for the default stream.
  * Calls on the same model share its scratch buffers: each call's work starts
  * after the previous call's (an event, also across streams), and calls from
- * several host threads are serialised by the model's lock.  n == 0 is a no-op. */
+ * several host threads are serialised by the model's lock.  n == 0 is a no-op.
+ * Two runs of one call give the same bits in 2D, in GWN_PREC_FP64 and in GWN_MODE_DIRECT
+ * (3D: while no list is full; repaired points to FP64 rounding); the 3D traversal in
+ * FP32 adds a point's terms in an order that varies, which moves values by their rounding
+ * (about 1e-7).  3D queries of at most 16 points keep one arithmetic and, but for
+ * rare ties, one order, so that values next to 0 (all points outside) repeat; they take up
+ * to 1 ms where 17 points take 0.15 ms. */
 gwn_status gwn_query(gwn_model model, const void* points, int32_t points_dtype, int32_t mem, size_t n,
                      double* out_w, int32_t* out_label, uint32_t* out_status, const gwn_query_opts* qopts,
                      void* stream);
@@ -229,6 +237,8 @@ gwn_status gwn_query(gwn_model model, const void* points, int32_t points_dtype, 
  *   Every call shares the one array: calls whose work overlaps on the GPU
  *   (concurrent streams, or threads that do not serialise their streams)
  *   race and must not be issued.
+ *   Two runs of one call give the same bits as long as no list of the scratch is full (3D: 7 pairs
+ *   a point next to their leaf, 3 in the FP64 near band, over 32,768 points).
  *   The model itself must have been built beforehand (gwn_build_* allocates). */
 gwn_status gwn_query_noalloc(gwn_model model, const void* points, int32_t points_dtype, size_t n, double* out_w,
                              int32_t* out_label, uint32_t* out_status, void* stream);

@@ -586,8 +586,10 @@ constexpr int kPacketWarpsPerSM = 112;
 // on 1.3M points of a 4.7k-leaf model.
 constexpr int kFastBlocks = 72, kEvalBlocks = 40;
 // Mean boundary curves per leaf from which two pairs per lane (k_pair_fast2, shared table
-// loads) pay: with 8, 3.43 -> 3.17 ms (1.3M points), 1.20 -> 1.10 ms (at the surface);
-// with 6 (the rings), whose runs fill fewer lanes of the wider warps, 2.69 -> 2.84 ms.
+// loads) pay: the loads it saves grow with the curves, what it loses -- runs of a leaf
+// fill fewer of the lanes -- does not.  Measured on two kinds of model only: with 8 curves 3.43 ->
+// 3.17 ms (1.3M points) and 1.20 -> 1.10 ms (at the surface), with 6 (rings) 2.69 -> 2.84 ms;
+// the line lies between them.
 constexpr size_t kPairedCurves = 7;
 constexpr int kQueryStats = 20;              // entries of gwn_last_query_stats
 
@@ -744,8 +746,9 @@ static gwn_status enqueue_chunk(gwn_model_s* m, const void* pts, int dtype, size
     if (p.precision == GWN_PREC_FP64 && m->dim == 3) {
         // the warp traversal and the FP64 pair list, for as many points at a time as
         // leave room for their pairs (a point whose pairs do not fit its share is still
-        // evaluated, by its own warp), the pairs' values summed in a fixed order.  One thread per point, each with its own branches and leaves,
-        // took 300 times as long (4001 points, 2.3k leaves: 1.49 s).
+        // evaluated, by its own warp), the pairs' values summed in a fixed order.  One thread per
+        // point, each with its own branches and leaves, took 150 times as long (4001
+        // points, 2.3k leaves: 1.48 s).
         const bool direct = p.mode == GWN_MODE_DIRECT;
         const bool all = direct && m->host.n_leaves <= kRepairPairCap;
         const size_t step = all ? std::max<size_t>(1, std::min(n, (size_t)(kRepairPairCap / m->host.n_leaves)))
@@ -859,8 +862,7 @@ static gwn_status enqueue_chunk(gwn_model_s* m, const void* pts, int dtype, size
             if (local) {
                 auto trav = m->stack_depth <= 64 ? k_trav3_local<64>
                                                  : m->stack_depth <= 96 ? k_trav3_local<96> : k_trav3_local<128>;
-                trav<<<1, B, 0, st>>>(m->tree, ws.spos, ni, nullptr, p.beta2, p.beta2_leaf, fw, p.work, nullptr, ws.olist,
-                                      p.kappa2);
+                trav<<<1, B, 0, st>>>(m->tree, ws.spos, ni, p.beta2, p.beta2_leaf, fw, p.work, ws.olist, p.kappa2);
             } else {
                 (o3 ? k_few_walk<true> : k_few_walk<false>)<<<1, 32, 0, st>>>(m->tree, ws.spos, ni, p.beta2, p.beta2_leaf,
                                                                             fw, p.work, ws.olist);
@@ -939,8 +941,7 @@ static gwn_status enqueue_chunk(gwn_model_s* m, const void* pts, int dtype, size
             } else if (local) {
                 auto trav = m->stack_depth <= 64 ? k_trav3_local<64>
                                                  : m->stack_depth <= 96 ? k_trav3_local<96> : k_trav3_local<128>;
-                trav<<<nb, B, 0, st>>>(m->tree, ws.spos, ni, nullptr, p.beta2, p.beta2_leaf, ws, p.work, nullptr,
-                                       ws.olist, p.kappa2);
+                trav<<<nb, B, 0, st>>>(m->tree, ws.spos, ni, p.beta2, p.beta2_leaf, ws, p.work, ws.olist, p.kappa2);
             } else {
                 packet_pass(none, false);
             }
@@ -1695,8 +1696,8 @@ gwn_status gwn_last_query_stats(gwn_model m, int64_t* out) {
     }
     for (int k = 0; k < kQueryStats; ++k) out[k] = 0;
     for (int k = 0; k < 4; ++k) out[k] = (int64_t)c[k];
-    out[2] = (int64_t)c[2];           // near-band (FP64) pairs over all rounds
-    out[3] = (int64_t)(c[6] + c[3]);  // points whose pairs overflowed in any round
+    out[2] = (int64_t)c[2];           // near-band (FP64) pairs of both passes
+    out[3] = (int64_t)(c[6] + c[3]);  // points whose pairs overflowed, in either pass
     for (int k = 0; k < 8; ++k) out[4 + k] = (int64_t)wk[k];
     out[14] = (int64_t)(c[8] + c[9]);  // pairs the full evaluator took (the rest came from the node tables)
     out[15] = (int64_t)wk[kWorkFastNodes];

@@ -135,14 +135,14 @@ struct DevTree {
     const float4* lhdr;
     const float4* lmom;
     const double* lhdr64;
-    const double* lmom64;
+    const double* lmom64;      // host execution (null on the device, which reads hmom64)
     // internal nodes
     const float4* hdr;         // (x0.x, x0.y, x0.z, r^2)
     const int2* child;
     const float4* chdr;        // 3D: 2 per internal node, the headers of its two children (hdr or lhdr)
     const float4* mom;         // kMom2Vec or kMom3Vec per node
     const double* hdr64;       // 4 per node
-    const double* mom64;       // kMom2F64 or kMom3F64 per node
+    const double* mom64;       // kMom2F64 or kMom3F64 per node; host execution, as lmom64
     // 2D leaves
     const float4* leaf2;       // kLeaf2Vec per leaf
     const double* leaf2_64;    // kLeaf2F64 per leaf

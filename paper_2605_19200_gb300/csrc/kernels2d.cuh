@@ -233,35 +233,4 @@ GWN_HD float query2_32(const DevTree& t, float qx, float qy, float beta2, uint32
     return w;
 }
 
-// Algorithm 1 in FP64 (repair pass); beta2 <= 0 evaluates every leaf directly.
-GWN_HD double query2_64(const DevTree& t, double qx, double qy, double beta2, uint32_t& st) {
-    double w = 0.0;
-    if (beta2 <= 0.0) {
-        for (int i = 0; i < t.n_leaves; ++i) w += leaf2_eval64(t, i, qx, qy, st);
-        return w;
-    }
-    int stack[kStack64];
-    int sp = 0;
-    int node = t.root;
-    while (true) {
-        if (node < 0) {
-            w += leaf2_eval64(t, ~node, qx, qy, st);
-        } else {
-            const double* h = t.hdr64 + (size_t)node * 4;
-            double rx = h[0] - qx, ry = h[1] - qy;
-            if (rx * rx + ry * ry > beta2 * h[3]) {
-                w += far2_eval<double>(t.mom64 + (size_t)node * kMom2F64, rx, ry);
-            } else {
-                int2 ch = t.child[node];
-                if (sp < kStack64) stack[sp++] = ch.y; else st |= GWN_QS_UNRESOLVED;
-                node = ch.x;
-                continue;
-            }
-        }
-        if (sp == 0) break;
-        node = stack[--sp];
-    }
-    return w;
-}
-
 }  // namespace gwn

@@ -51,7 +51,6 @@ constexpr double kRatio64Exact = 0.5;
 // the warp evaluator (leaf3_warp64<4>) takes 4-point panels at half these ratios,
 // which keeps the same Bernstein-ellipse margin per panel with half the nodes
 constexpr double kRatio64BandW4 = 0.75;
-constexpr double kRatio64RepairW4 = 0.5;
 
 // binomial coefficients and the 8-point Gauss-Legendre rule on [0, 1]: device
 // constant memory, with host mirrors for host-side execution

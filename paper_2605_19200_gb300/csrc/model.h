@@ -53,7 +53,7 @@ struct gwn_model_s {
     gwn::Workspace ws{};
     static constexpr int kMaxProfChunks = 32;
     // per chunk: before and after the traversal, before the table kernel,
-    // after the full evaluator, between the two (round 0 of each chunk)
+    // after the full evaluator, between the two (the first pass of each chunk)
     cudaEvent_t ev[kMaxProfChunks][5] = {};
     int prof_chunks = 0;
     bool profiled = false;

@@ -239,7 +239,7 @@ constexpr int kPairBuf = 128;  // (point, leaf) pairs buffered per warp in share
 // write a warp's buffered pairs (n of them, warp-uniform) to the pair list with
 // one atomic and coalesced stores.  If the list is full, the lanes that own the
 // entries which did not fit are added to `ovf` (every lane gets the same mask);
-// their points skip the pair pass and are traversed again in the next round.
+// their points skip the pair pass and are evaluated again without the list (k_wide3).
 __device__ __forceinline__ void flush_warp_pairs(const int2* buf, const unsigned char* own, int n, const Workspace& ws,
                                                  unsigned& ovf) {
     const unsigned full = 0xffffffffu;
@@ -492,9 +492,9 @@ __global__ void __launch_bounds__(32, 28) k_trav3(DevTree t, const float4* spos,
 // sharing k_trav3's body cost the plain traversal 4 % (9.16 -> 9.51 ms on a
 // 2M-query model) at the same register count.
 template <int STACK>
-__global__ void __launch_bounds__(128) k_trav3_local(DevTree t, const float4* spos, int n, const int* list,
-                                               float beta2, float beta2l, Workspace ws, unsigned long long* work,
-                                               const int* n_dev, int* olist_out, float kappa2) {
+__global__ void __launch_bounds__(128) k_trav3_local(DevTree t, const float4* spos, int n, float beta2, float beta2l,
+                                                     Workspace ws, unsigned long long* work, int* olist_out,
+                                                     float kappa2) {
     __shared__ int2 sstk[4][STACK];
     __shared__ int2 sbuf[4][kPairBuf];
     __shared__ unsigned char sown[4][kPairBuf];
@@ -506,11 +506,9 @@ __global__ void __launch_bounds__(128) k_trav3_local(DevTree t, const float4* sp
     unsigned char* own = sown[threadIdx.x >> 5];
     int* lst = slocal[threadIdx.x >> 5];
     WorkLocal wl = {};
-    if (n_dev) n = *n_dev;
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n_dev && blockIdx.x * blockDim.x >= n) return;  // whole block past the list
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const bool active = i < n;
-    const int qi = active ? (list ? list[i] : i) : 0;
+    const int qi = active ? i : 0;
     float q[3] = {0, 0, 0};
     if (active) {
         const float4 p = spos[qi];
@@ -695,7 +693,7 @@ namespace gwn {
 // query one after the other are the longest chain.
 // A query costs about twice the instructions of its share of a packet, with 64
 // times the warps.
-// list, n_dev: as in k_trav3 (n_dev: the list's length on the device); again: as in
+// list: the points to take (null: all n), n_dev: their number on the device; again: as in
 // k_trav3, without it a dense chunk's leaves take beta2
 constexpr int kWideStack = 768;  // stack_take
 template <bool O3, bool COUNT, bool LIST>
@@ -862,8 +860,8 @@ __global__ void __launch_bounds__(128) k_wide3(DevTree t, const float4* spos, in
     if (COUNT) flush_work(wl, work);
 }
 
-// points whose pairs still overflowed after the last round: whole traversal
-// again, leaves in place
+// points with a pair that did not fit a list in the last pass: whole traversal again, leaves in
+// place (at beta2: tighter than the far test of the other points' leaves)
 __global__ void __launch_bounds__(128) k_overflow3(DevTree t, const float4* spos, float beta2, Workspace ws,
                                                    const int* list, long long* near = nullptr) {
     int cnt = ws.counters[3];
@@ -1525,9 +1523,9 @@ __global__ void k_next_round(Workspace ws) {
     if (threadIdx.x == 0) {
         ws.counters[5] = ws.counters[3];
         ws.counters[6] += ws.counters[3];
-        ws.counters[9] += ws.counters[8];  // of which the full evaluator took
+        ws.counters[9] += ws.counters[8];  // pairs the full evaluator took
         ws.counters[3] = 0;
-        ws.counters[0] = 0;  // the near-band list (counters[2]) spans all rounds
+        ws.counters[0] = 0;  // the near-band list (counters[2]) spans both passes
         ws.counters[8] = 0;
     }
 }
